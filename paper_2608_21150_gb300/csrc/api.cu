@@ -280,7 +280,7 @@ bool terrain_complete(const TerrT<T>& t) {
 }
 
 bool work_complete(const DevWork& w) {
-  const void* p[] = {w.div_m, w.div_t, w.rho_p, w.theta_p, w.w_p, w.pex, w.col, w.zbl, w.diag, w.flag};
+  const void* p[] = {w.div_m, w.div_t, w.rho_p, w.theta_p, w.w_p, w.pex, w.col, w.diag, w.flag};
   for (const void* q : p)
     if (!q) return false;
   return true;
@@ -306,7 +306,7 @@ int autotune(icon_dycore* d) {
   // Candidates: threads per CTA (128, 256, 512) x tile shape (one thread per
   // (point, level), or one warp per point with its lanes over the levels) for
   // the stencil kernels; levels per shared-memory chunk (8, 6, 4) for the
-  // column solve.  Each candidate runs kReps steps; a kernel's time is the
+  // column solve's predictor and corrector (its wide form).  Each candidate runs kReps steps; a kernel's time is the
   // smallest of its per-step sums, so a single noisy sample cannot decide.
   constexpr int kReps = 3;
   const int cand[3] = {128, 256, 512};
@@ -315,13 +315,13 @@ int autotune(icon_dycore* d) {
   std::vector<double> t(kNumStencils * 2 * 3, kInf);
   auto tk = [&](int k, int sh, int ci) -> double& { return t[((size_t)k * 2 + sh) * 3 + ci]; };
   const int col_cand[3] = {8, 6, 4};
-  double col_t[3] = {kInf, kInf, kInf};
+  double col_t[2][3] = {{kInf, kInf, kInf}, {kInf, kInf, kInf}};  // predictor, corrector
   auto run = [&](int ci, int shape, int kc, bool stencils) -> int {
     for (int k = 0; k < kNumStencils; ++k) {
       d->en.threads[k] = cand[ci];
       d->en.shape[k] = shape;
     }
-    d->en.col_kc = kc;
+    d->en.col_kc[0] = d->en.col_kc[1] = kc;
     Prof prof;
     g_prof = &prof;
     enqueue_op(d, 0, st, d->stream);
@@ -329,13 +329,13 @@ int autotune(icon_dycore* d) {
     CUDA_TRY(cudaGetLastError());
     CUDA_TRY(cudaStreamSynchronize(d->stream));
     std::vector<double> sum(kNumStencils, 0.0);
-    double col = 0.0;
+    double col[2] = {0.0, 0.0};
     for (const auto& r : prof.recs) {
       float ms = 0.f;
       CUDA_TRY(cudaEventElapsedTime(&ms, r.e0, r.e1));
       std::string nm = r.name;
       if (nm.compare(0, 9, "sn_column") == 0) {
-        col += ms;
+        col[nm.compare(0, 14, "sn_column_corr") == 0 ? 1 : 0] += ms;
         continue;
       }
       if (nm.compare(0, 15, "sn_cell_fluxsum") == 0) nm = "sn_cell_fluxdiv" + nm.substr(15);  // same id
@@ -349,15 +349,16 @@ int autotune(icon_dycore* d) {
       for (int k = 0; k < kNumStencils; ++k)
         if (sum[k] > 0.0) tk(k, shape, ci) = std::min(tk(k, shape, ci), sum[k]);
     for (int j = 0; j < 3; ++j)
-      if (col_cand[j] == kc) col_t[j] = std::min(col_t[j], col);
+      if (col_cand[j] == kc)
+        for (int i = 0; i < 2; ++i) col_t[i][j] = std::min(col_t[i][j], col[i]);
     return ICON_OK;
   };
   if (rc == ICON_OK) rc = run(1, 0, 8, false);  // warm-up (module load, first-touch)
-  if (rc == ICON_OK) col_t[0] = kInf;
+  if (rc == ICON_OK) col_t[0][0] = col_t[1][0] = kInf;
   for (int shape = 0; shape < 2; ++shape)
     for (int ci = 0; ci < 3; ++ci)
       for (int r = 0; r < kReps && rc == ICON_OK; ++r) rc = run(ci, shape, 8, true);
-  for (int j = 1; j < 3; ++j)
+  for (int j = 1; j < 3 && !d->en.col_narrow; ++j)
     for (int r = 0; r < kReps && rc == ICON_OK; ++r) rc = run(1, 0, col_cand[j], false);
   for (double* p : {st.vn, st.w, st.rho, st.exner, st.theta_v, st.exner_pr})
     if (p) cudaFree(p);
@@ -374,10 +375,12 @@ int autotune(icon_dycore* d) {
     // only va_edge_pre, va_cell_w, sn_cell_div and sn_edge_corr have both shapes
     d->en.shape[k] = (k == 0 || k == 3 || k == 6 || k == 8) ? best_sh : -1;
   }
-  int best_kc = 0;
-  for (int j = 1; j < 3; ++j)
-    if (col_t[j] < col_t[best_kc]) best_kc = j;
-  d->en.col_kc = col_cand[best_kc];
+  for (int i = 0; i < 2; ++i) {
+    int best_kc = 0;
+    for (int j = 1; j < 3; ++j)
+      if (col_t[i][j] < col_t[i][best_kc]) best_kc = j;
+    d->en.col_kc[i] = col_cand[best_kc];
+  }
   return ICON_OK;
 }
 
@@ -804,8 +807,7 @@ int create_dycore(const icon_grid_t* grid, int nlev, const double* z_ifc, const 
   w.theta_p = A.alloc<double>(cf);
   w.w_p = A.alloc<double>(ch);
   w.pex = A.alloc<double>(cf);
-  w.col = A.alloc<double>(7 * ch);
-  w.zbl = A.alloc<double>(ch);
+  w.col = A.alloc<double>(8 * (cf + (size_t)kColWide * nlev));  // whole groups of columns
   w.diag = A.alloc<double>(diag_partials(nc));
   w.flag = A.alloc<int>(1);
   if (A.status == cudaSuccess) {
@@ -842,7 +844,7 @@ int create_dycore(const icon_grid_t* grid, int nlev, const double* z_ifc, const 
     }
   }
   for (int k = 0; k < kNumStencils; ++k) en.threads[k] = 256;
-  en.col_kc = 4;
+  en.col_narrow = p->column_chunk == 0 && narrow_columns(nc);
   if (p->autotune) {
     int rc = autotune(d);
     if (rc != ICON_OK) {
@@ -852,7 +854,7 @@ int create_dycore(const icon_grid_t* grid, int nlev, const double* z_ifc, const 
       return rc;
     }
   }
-  if (p->column_chunk) en.col_kc = p->column_chunk;
+  if (p->column_chunk) en.col_kc[0] = en.col_kc[1] = p->column_chunk;
   *out = d;
   return ICON_OK;
 }
@@ -1440,7 +1442,13 @@ int icon_dycore_launch_config(const icon_dycore_t* d, char* buf, int32_t len) {
     if (d->en.shape[k] >= 0) s += d->en.shape[k] ? "w" : "t";
     s += ",";
   }
-  s += "column_threads=64;column_chunk=" + std::to_string(d->en.col_kc);
+  s += "column_columns=" + std::to_string(d->en.col_narrow ? kColNarrow : kColWide) + ";column_chunk=";
+  if (d->en.col_narrow)
+    s += "8";
+  else if (d->en.col_kc[0] == d->en.col_kc[1])
+    s += std::to_string(d->en.col_kc[0]);
+  else
+    s += std::to_string(d->en.col_kc[0]) + "/" + std::to_string(d->en.col_kc[1]);
   std::snprintf(buf, (size_t)len, "%s", s.c_str());
   return ICON_OK;
 }

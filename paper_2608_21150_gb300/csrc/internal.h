@@ -236,8 +236,7 @@ struct DevWork {
   double *rho_p, *theta_p;                // cells: predicted state (the corrector's time averages)
   double* w_p;                            // cells, half levels
   double* pex;   // cells: extrapolated exner perturbation (FP64, or double-word pairs in mixed mode)
-  double* col;   // level-major [k][c] scratch: 7 planes of (nlev+1)*nc: cp, rp, rho*, pr*, rho_ic, alpha, eos
-  double* zbl;   // level-major zb [(nlev+1)*nc], predictor -> corrector
+  double* col;   // column solve scratch [level][group of columns][8 planes][column] (column_kernel.cuh)
   double* diag;  // diagnostics: partial column-mass sums
   int* flag;     // diagnostics: non-finite flag
 };

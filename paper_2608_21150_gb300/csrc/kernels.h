@@ -68,6 +68,14 @@ struct Ctx {
 // The fused velocity-advection kernel's shared-memory limit for these patches.
 cudaError_t init_va_fused(const VaPatchT& pt);
 
+// Columns per CTA of the column solve: 32 (a warp's lanes are 32 columns, the
+// elimination runs at full width) once they give every SM four CTAs; below
+// that 16, so that a small grid spreads over more SMs.  Measured, predictor,
+// wide (chunks of 8) against narrow: FP64 R2B2 L30 35 / 27 us, R2B3 L31 49 /
+// 43, R2B4 L65 206 / 214; mixed R2B3 L31 30 / 26, R2B4 L65 103 / 127.
+constexpr int kColWide = 32, kColNarrow = 16;
+inline bool narrow_columns(int nc) { return nc < 4 * 152 * kColWide; }
+
 // Device-side state of one dycore: FP64 factors and column-solve work, the
 // FP32 mirrors (mixed mode) and the stencil context of the active mode.
 // The mixed modes (FP32 stencils) differ only in the column solve's arithmetic.
@@ -84,14 +92,15 @@ struct Engine {
   Ctx<double> c64{};
   Ctx<float> c32{};
   // launch configuration picked by the autotuner: threads per CTA of each
-  // stencil kernel (by kernel id) and the level-chunk depth of the column solve
+  // stencil kernel (by kernel id), and the level-chunk depth of the column solve
   int threads[32] = {};
   // tile shape of the two-shape kernels (va_edge_pre, va_cell_w, sn_cell_div,
   // sn_edge_corr): 1 one warp per point (lanes over its levels), 0 one thread
   // per (point, level); -1 the compute type's default
   int shape[32] = {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1,
                    -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1};
-  int col_kc = 4;
+  int col_kc[2] = {8, 4};   // the column solve's level chunk: predictor, corrector
+  bool col_narrow = false;  // the column solve's form for small grids
   bool terrain = false;  // per-column heights: the terrain forms of the kernels
   // Host-array steps: when set, the first substep waits on this event right
   // after its predictor's velocity tendencies (which read only vn and w), so

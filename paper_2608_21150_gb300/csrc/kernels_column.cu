@@ -59,9 +59,16 @@ constexpr size_t kNoallocStride = 512;                 // doubles per vertical-m
 constexpr size_t kNoallocCoef = 10752;                 // doubles of the vertical-metric section
 constexpr size_t kNoallocLevHL = 6400;                 // offset of the double-word level table
 constexpr size_t kNoallocDoubles = (size_t)8 << 20;    // 64 MiB in total
-constexpr size_t kNoallocPlanes = 8;                   // 7 Thomas planes + zb
+constexpr size_t kNoallocPlanes = 8;                   // kScratchPlanes
 constexpr size_t kNoallocMaxPoints = (kNoallocDoubles - kNoallocCoef) / kNoallocPlanes;
 static_assert(kNoallocMaxPoints == 1047232, "the limit stated in icon_dycore.h");
+static_assert(kNoallocPlanes == kScratchPlanes, "planes of the column solve's scratch");
+// The scratch holds whole groups of columns on nlev levels: at most (n_cols +
+// 15) nlev column-levels in the narrow form, which 15 nlev <= n_cols keeps
+// within n_cols (nlev + 1) (fewer columns than that stay below the limit), and (n_cols + 31) nlev in the wide one (n_cols >= 19 456, so nlev <= 52).
+static_assert(kColNarrow == 16 && 15 * (size_t)kNoallocMaxLev * (kNoallocMaxLev + 1) < kNoallocMaxPoints &&
+                  31 * (kNoallocMaxPoints / (4 * 152 * kColWide)) <= 4 * 152 * kColWide,
+              "the groups' spare columns fit");
 static_assert(8 * kNoallocStride + 8 * (kNoallocMaxLev + 1) <= kNoallocLevHL, "column coefficients fit");
 static_assert(kNoallocLevHL + 16 * (kNoallocMaxLev + 1) <= kNoallocCoef, "level table fits");
 
@@ -85,85 +92,93 @@ __device__ __forceinline__ void split_pair(double x, float* out) {
 // The vertical metrics, reference state, Rayleigh factors, column
 // coefficients and double-word level table of icon_dycore_create, written
 // into the metric section of the static array (every slot the column kernel
-// reads, zeros included, so nothing is left from an earlier call).  One
-// thread: about nlev sequential levels of scalar work.
-__global__ void noalloc_metrics(NoallocSetup q, double* base) {
-  if (blockIdx.x != 0 || threadIdx.x != 0) return;
-  const int nlev = q.nlev;
-  double* dz = base;
-  double* inv_dz = base + kNoallocStride;
-  double* inv_dzh = base + 2 * kNoallocStride;
-  double* wgt = base + 3 * kNoallocStride;
-  double* th_ref = base + 4 * kNoallocStride;
-  double* ex_ref = base + 5 * kNoallocStride;
-  double* dref = base + 6 * kNoallocStride;
-  double* ray = base + 7 * kNoallocStride;
-  double* colc = base + 8 * kNoallocStride;
-  float* lev = reinterpret_cast<float*>(base + kNoallocLevHL);
+// reads, zeros included, so nothing is left from an earlier call).  One CTA, a
+// thread per half level; only the reference exner, summed up from the ground,
+// is sequential (one subtraction a level).  One thread walking all levels
+// took about 400 of the call's 950 us at 90 levels.
+constexpr int kNoallocThreads = 288;
+static_assert(kNoallocThreads > kNoallocMaxLev, "a thread per half level");
+__global__ void __launch_bounds__(kNoallocThreads) noalloc_metrics(NoallocSetup q, double* base) {
+  __shared__ double s_th[kNoallocMaxLev], s_ex[kNoallocMaxLev], s_drop[kNoallocMaxLev + 1];
+  const int nlev = q.nlev, k = threadIdx.x;
   const double* z = q.z_ifc;
   const double H = q.cpd * q.ref_T0 / q.grav;
-  for (int k = 0; k < nlev; ++k) {
-    const double zm = 0.5 * (z[k] + z[k + 1]);
-    dz[k] = z[k] - z[k + 1];
-    inv_dz[k] = 1.0 / dz[k];
-    th_ref[k] = q.ref_T0 * exp(zm / H);
+  const bool full = k < nlev, half = k <= nlev, inner = k >= 1 && k < nlev;
+  double dz = 0.0;
+  if (full) {
+    dz = z[k] - z[k + 1];
+    s_th[k] = q.ref_T0 * exp(0.5 * (z[k] + z[k + 1]) / H);
   }
-  for (int k = 0; k <= nlev; ++k) {
-    inv_dzh[k] = 0.0;
-    wgt[k] = 0.0;
-    dref[k] = 0.0;
-  }
-  for (int k = 1; k < nlev; ++k) {
+  __syncthreads();
+  double inv_dzh = 0.0, wgt = 0.0, th_ic = 0.0;
+  if (inner) {
     const double zu = 0.5 * (z[k - 1] + z[k]), zl = 0.5 * (z[k] + z[k + 1]);
-    inv_dzh[k] = 1.0 / (zu - zl);
-    wgt[k] = (z[k] - zl) / (zu - zl);
+    inv_dzh = 1.0 / (zu - zl);
+    wgt = (z[k] - zl) / (zu - zl);
+    th_ic = wgt * s_th[k - 1] + (1.0 - wgt) * s_th[k];
+    s_drop[k] = q.grav * (zu - zl) / (q.cpd * th_ic);
   }
-  ex_ref[nlev - 1] = exp(-0.5 * (z[nlev - 1] + z[nlev]) / H);
-  for (int k = nlev - 1; k >= 1; --k) {
-    const double zu = 0.5 * (z[k - 1] + z[k]), zl = 0.5 * (z[k] + z[k + 1]);
-    const double th_ic = wgt[k] * th_ref[k - 1] + (1.0 - wgt[k]) * th_ref[k];
-    ex_ref[k - 1] = ex_ref[k] - q.grav * (zu - zl) / (q.cpd * th_ic);
-  }
-  for (int k = 1; k < nlev; ++k) dref[k] = (ex_ref[k - 1] - ex_ref[k]) * inv_dzh[k];
-  for (int k = 0; k <= nlev; ++k) {
-    ray[k] = 1.0;
-    if (q.rayleigh_coeff > 0.0 && z[k] > q.damp_height) {
-      const double sn = sin(0.5 * 3.141592653589793 * (z[k] - q.damp_height) / (z[0] - q.damp_height));
-      ray[k] = 1.0 / (1.0 + q.dt_s * q.rayleigh_coeff * sn * sn);
+  __syncthreads();
+  if (k == 0) {
+    double e = exp(-0.5 * (z[nlev - 1] + z[nlev]) / H);
+    s_ex[nlev - 1] = e;
+    for (int j = nlev - 1; j >= 1; --j) {
+      e = e - s_drop[j];
+      s_ex[j - 1] = e;
     }
   }
-  for (int k = 0; k <= nlev; ++k) {
-    double* cf = colc + 8 * (size_t)k;
-    for (int j = 0; j < 8; ++j) cf[j] = 0.0;
-    if (k < nlev) {
-      cf[0] = q.dt_s * q.rd_o_cvd / dz[k];
-      cf[1] = q.dt_s * (1.0 - q.beta) / dz[k];
-      cf[2] = q.dt_s * q.beta / dz[k];
-    }
-    if (k >= 1 && k < nlev) {
-      cf[4] = q.dt_s * q.cpd * dref[k];
-      cf[5] = q.dt_s * q.cpd * q.beta * inv_dzh[k];
-      cf[6] = wgt[k];
-      cf[7] = 1.0 - wgt[k];
-      cf[3] = cf[6] * th_ref[k - 1] + cf[7] * th_ref[k];
-    }
-    // the double-word table: colc, then exner_ref, theta_ref, dz, ray_fac
-    // (no rho offset: this entry point's inputs are FP64)
-    float* r = lev + 32 * (size_t)k;
-    for (int j = 0; j < 32; ++j) r[j] = 0.0f;
-    for (int j = 0; j < 8; ++j) split_pair(cf[j], r + 2 * j);
-    if (k < nlev) {
-      split_pair(ex_ref[k], r + 16);
-      split_pair(th_ref[k], r + 18);
-      split_pair(dz[k], r + 20);
-    }
-    split_pair(ray[k], r + 22);
+  __syncthreads();
+  if (!half) return;
+  const double dref = inner ? (s_ex[k - 1] - s_ex[k]) * inv_dzh : 0.0;
+  double ray = 1.0;
+  if (q.rayleigh_coeff > 0.0 && z[k] > q.damp_height) {
+    const double sn = sin(0.5 * 3.141592653589793 * (z[k] - q.damp_height) / (z[0] - q.damp_height));
+    ray = 1.0 / (1.0 + q.dt_s * q.rayleigh_coeff * sn * sn);
   }
+  if (full) {
+    base[k] = dz;
+    base[kNoallocStride + k] = 1.0 / dz;
+    base[4 * kNoallocStride + k] = s_th[k];
+    base[5 * kNoallocStride + k] = s_ex[k];
+  }
+  base[2 * kNoallocStride + k] = inv_dzh;
+  base[3 * kNoallocStride + k] = wgt;
+  base[6 * kNoallocStride + k] = dref;
+  base[7 * kNoallocStride + k] = ray;
+  double cf[8] = {};
+  if (full) {
+    cf[0] = q.dt_s * q.rd_o_cvd / dz;
+    cf[1] = q.dt_s * (1.0 - q.beta) / dz;
+    cf[2] = q.dt_s * q.beta / dz;
+  }
+  if (inner) {
+    cf[4] = q.dt_s * q.cpd * dref;
+    cf[5] = q.dt_s * q.cpd * q.beta * inv_dzh;
+    cf[6] = wgt;
+    cf[7] = 1.0 - wgt;
+    cf[3] = th_ic;
+  }
+  double* colc = base + 8 * kNoallocStride + 8 * (size_t)k;
+  for (int j = 0; j < 8; ++j) colc[j] = cf[j];
+  // the double-word table: colc, then exner_ref, theta_ref, dz, ray_fac
+  // (no rho offset: this entry point's inputs are FP64)
+  float* r = reinterpret_cast<float*>(base + kNoallocLevHL) + 32 * (size_t)k;
+  for (int j = 0; j < 32; ++j) r[j] = 0.0f;
+  for (int j = 0; j < 8; ++j) split_pair(cf[j], r + 2 * j);
+  if (full) {
+    split_pair(s_ex[k], r + 16);
+    split_pair(s_th[k], r + 18);
+    split_pair(dz, r + 20);
+  }
+  split_pair(ray, r + 22);
 }
 
 constexpr int kNoallocMaxDevices = 64;
 std::mutex g_noalloc_mutex;
 double* g_noalloc_ptr[kNoallocMaxDevices] = {};
+
+using NoallocWide = ColForm<double, 8, kColWide, 2, true, false>;
+using NoallocNarrow = ColForm<double, 8, kColNarrow, 1, true, false>;
 
 // Once per device, with that device current: the device address of the
 // static array (its host-side name is only a stand-in) and the kernel's
@@ -180,10 +195,13 @@ int noalloc_setup(double** out) {
     e = cudaGetSymbolAddress((void**)&ptr, g_noalloc_scratch);
     if (e != cudaSuccess)
       return report_error(ICON_ERR_CUDA, std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e));
-    e = cudaFuncSetAttribute(sn_column_tiled<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(sn_column_tiled<double, true, kKC, dws>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)kSmem);
+    auto set = [&](auto kernel, size_t bytes) {
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    set(sn_column<double, double, 8, kColWide, 2, -1, false, true>, NoallocWide::bytes);
+    set(sn_column<double, dws, 8, kColWide, 2, -1, false, true>, NoallocWide::bytes);
+    set(sn_column<double, double, 8, kColNarrow, 1, -1, false, true>, NoallocNarrow::bytes);
+    set(sn_column<double, dws, 8, kColNarrow, 1, -1, false, true>, NoallocNarrow::bytes);
     if (e != cudaSuccess)
       return report_error(ICON_ERR_CUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));
     g_noalloc_ptr[dev] = ptr;
@@ -264,7 +282,7 @@ extern "C" int icon_column_solve_noalloc(int32_t n_cols, int32_t nlev, const dou
   if (rc != ICON_OK) return rc;
   cudaStream_t stream = static_cast<cudaStream_t>(p->stream);
   // the metrics into the static array, on the device, from the by-value block
-  noalloc_metrics<<<1, 32, 0, stream>>>(q, base);
+  noalloc_metrics<<<1, kNoallocThreads, 0, stream>>>(q, base);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return report_error(ICON_ERR_CUDA, std::string(fn) + cudaGetErrorString(e));
   DevVert v{};
@@ -298,16 +316,27 @@ extern "C" int icon_column_solve_noalloc(int32_t n_cols, int32_t nlev, const dou
   a.div_m = div_m;
   a.div_t = div_t;
   a.col = base + kNoallocCoef;
-  a.zbl = a.col + 7 * points;
   a.w_o = w_new;
   a.rho_o = rho_new;
   a.exner_o = exner_new;
   a.theta_o = theta_new;
-  const unsigned blocks = (unsigned)((n_cols + kCW - 1) / kCW);
-  if (p->precision == ICON_PREC_MIXED)  // the mixed mode's double-word FP32 arithmetic
-    sn_column_tiled<double, true, kKC, dws><<<blocks, kCW, kSmem, stream>>>(n_cols, v, s, corr ? 1 : 0, a);
-  else
-    sn_column_tiled<double, true><<<blocks, kCW, kSmem, stream>>>(n_cols, v, s, corr ? 1 : 0, a);
+  const bool dw = p->precision == ICON_PREC_MIXED;  // the mixed mode's double-word FP32 arithmetic
+  const int corrector = corr ? 1 : 0;
+  if (narrow_columns(n_cols)) {
+    using F = NoallocNarrow;
+    const unsigned blocks = (unsigned)((n_cols + kColNarrow - 1) / kColNarrow);
+    if (dw)
+      sn_column<double, dws, 8, kColNarrow, 1, -1, false, true><<<blocks, F::NT, F::bytes, stream>>>(n_cols, v, s, corrector, a);
+    else
+      sn_column<double, double, 8, kColNarrow, 1, -1, false, true><<<blocks, F::NT, F::bytes, stream>>>(n_cols, v, s, corrector, a);
+  } else {
+    using F = NoallocWide;
+    const unsigned blocks = (unsigned)((n_cols + kColWide - 1) / kColWide);
+    if (dw)
+      sn_column<double, dws, 8, kColWide, 2, -1, false, true><<<blocks, F::NT, F::bytes, stream>>>(n_cols, v, s, corrector, a);
+    else
+      sn_column<double, double, 8, kColWide, 2, -1, false, true><<<blocks, F::NT, F::bytes, stream>>>(n_cols, v, s, corrector, a);
+  }
   e = cudaGetLastError();
   if (e != cudaSuccess) return report_error(ICON_ERR_CUDA, std::string(fn) + cudaGetErrorString(e));
   if (p->synchronous) {
