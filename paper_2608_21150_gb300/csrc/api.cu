@@ -306,8 +306,9 @@ int autotune(icon_dycore* d) {
   // Candidates: threads per CTA (128, 256, 512) x tile shape (one thread per
   // (point, level), or one warp per point with its lanes over the levels) for
   // the stencil kernels; levels per shared-memory chunk (8, 6, 4) for the
-  // column solve's predictor and corrector (its wide form).  Each candidate runs kReps steps; a kernel's time is the
-  // smallest of its per-step sums, so a single noisy sample cannot decide.
+  // column solve's predictor and corrector (its wide form).  Each candidate
+  // runs kReps steps; a kernel's time is the smallest of its per-step sums, so
+  // a single noisy sample cannot decide.
   constexpr int kReps = 3;
   const int cand[3] = {128, 256, 512};
   constexpr double kInf = 1e300;
@@ -372,8 +373,9 @@ int autotune(icon_dycore* d) {
           best_ci = ci;
         }
     d->en.threads[k] = cand[best_ci];
-    // only va_edge_pre, va_cell_w, sn_cell_div and sn_edge_corr have both shapes
-    d->en.shape[k] = (k == 0 || k == 3 || k == 6 || k == 8) ? best_sh : -1;
+    // only va_edge_pre, va_cell_w, sn_cell_div (FP64) and sn_edge_corr have both shapes
+    const bool two = k == 8 || (!is_mixed(d->en.precision) && (k == 0 || k == 3 || k == 6));
+    d->en.shape[k] = two ? best_sh : -1;
   }
   for (int i = 0; i < 2; ++i) {
     int best_kc = 0;
@@ -565,10 +567,19 @@ int create_dycore(const icon_grid_t* grid, int nlev, const double* z_ifc, const 
 
   const size_t ef = (size_t)ne * nlev, eh = (size_t)ne * (nlev + 1);
   const size_t cf = (size_t)nc * nlev, ch = (size_t)nc * (nlev + 1);
-  const size_t vf = (size_t)nv * nlev, vh = (size_t)nv * (nlev + 1);
+  // row strides of the stencil fields (VertT): FP32 rows padded to whole quads of levels
+  const int ld32 = (nlev + 4) / 4 * 4;
   auto build_ctx = [&](auto& x, auto tag) {
     using T = decltype(tag);
+    constexpr bool f32 = std::is_same<T, float>::value;
+    const size_t ldf = f32 ? ld32 : nlev, ldh = f32 ? ld32 : nlev + 1;
+    const size_t ef = ne * ldf, eh = ne * ldh, cf = nc * ldf, ch = nc * ldh, vf = nv * ldf, vh = nv * ldh;
     auto up = [&](const std::vector<double>& src) { return A.upload(std::vector<T>(src.begin(), src.end())); };
+    auto up_levels = [&](const std::vector<double>& src) {
+      std::vector<T> q(src.begin(), src.end());
+      q.resize(std::max(q.size(), ldh), T(0));
+      return A.upload(q);
+    };
     GridT<T>& g = x.g;
     const DevGrid& g0 = grid->dev;
     g.nc = nc;
@@ -615,18 +626,20 @@ int create_dycore(const icon_grid_t* grid, int nlev, const double* z_ifc, const 
     g.mean_area = (T)h.mean_area;
     VertT<T>& vt = x.v;
     vt.nlev = nlev;
-    vt.inv_dz = up(inv_dz);
-    vt.inv_dzh = up(inv_dzh);
+    vt.ldf = (int)ldf;
+    vt.ldh = (int)ldh;
+    vt.inv_dz = up_levels(inv_dz);
+    vt.inv_dzh = up_levels(inv_dzh);
     {
       std::vector<double> q(inv_dz), qh(inv_dzh);
       for (double& x : q) x *= 0.25;
       for (double& x : qh) x *= 0.5;
-      vt.qdz = up(q);
-      vt.qdzh = up(qh);
+      vt.qdz = up_levels(q);
+      vt.qdzh = up_levels(qh);
     }
-    vt.wgt = up(wgt);
-    vt.theta_ref = up(d->theta_ref);
-    vt.rho_ref = up(rho_ref);
+    vt.wgt = up_levels(wgt);
+    vt.theta_ref = up_levels(d->theta_ref);
+    vt.rho_ref = up_levels(rho_ref);
     vt.exner_ref = v.exner_ref;
     ScalT<T>& st = x.s;
     st.dt_s = (T)s.dt_s;
@@ -744,11 +757,8 @@ int create_dycore(const icon_grid_t* grid, int nlev, const double* z_ifc, const 
       vp.own_w = A.upload(own_w);
     }
     Mirrors& m = en.m;
-    m.vn = A.alloc<float>(ef);
-    m.w = A.alloc<float>(ch);
-    m.rho = A.alloc<float>(cf);
-    m.th = A.alloc<float>(cf);
-    m.w_p = A.alloc<float>(ch);
+    m.vn = A.alloc<float>((size_t)ne * ld32);
+    for (float** q : {&m.w, &m.rho, &m.th, &m.w_p}) *q = A.alloc<float>((size_t)nc * ld32);
   }
 
   // terrain: per-column reference state and column-solve table, and the
@@ -767,24 +777,27 @@ int create_dycore(const icon_grid_t* grid, int nlev, const double* z_ifc, const 
     }
     auto build_terr = [&](auto& x, auto tag) {
       using T = decltype(tag);
-      auto up = [&](const std::vector<double>& src) { return A.upload(std::vector<T>(src.begin(), src.end())); };
+      const size_t ldf = x.v.ldf, ldh = x.v.ldh;
+      // rows of nk levels, times f, at the stride ld
+      auto up = [&](const std::vector<double>& src, size_t nk, size_t ld, double f = 1.0) {
+        const size_t rows = src.size() / nk;
+        std::vector<T> q(rows * ld, T(0));
+        for (size_t r = 0; r < rows; ++r)
+          for (size_t k = 0; k < nk; ++k) q[r * ld + k] = (T)(src[r * nk + k] * f);
+        return A.upload(q);
+      };
+      const size_t nf = nlev, nh = nlev + 1;
       TerrT<T>& t = x.tr;
-      t.wgt_e = up(ht.wgt_e);
-      std::vector<double> q(ht.inv_dz_e);
-      for (double& x : q) x *= 0.25;
-      t.qdz_e = up(q);
-      t.ddxn_ifc = up(ht.ddxn_ifc);
-      t.ddxt_ifc = up(ht.ddxt_ifc);
-      std::vector<double> cpd_ddxn(ht.ddxn_mc);
-      for (double& x : cpd_ddxn) x *= p->cpd;
-      t.ddxn_mc = up(cpd_ddxn);
-      std::vector<double> qh(ht.inv_dzh_c);
-      for (double& x : qh) x *= 0.5;
-      t.qdzh_c = up(qh);
-      t.inv_dzm_c = up(ht.inv_dzm_c);
-      t.fx_ratio = up(ht.fx_ratio);
-      t.wcc0 = A.template alloc<T>(ch);
-      t.wcc1 = A.template alloc<T>(ch);
+      t.wgt_e = up(ht.wgt_e, nh, ldh);
+      t.qdz_e = up(ht.inv_dz_e, nf, ldf, 0.25);
+      t.ddxn_ifc = up(ht.ddxn_ifc, nh, ldh);
+      t.ddxt_ifc = up(ht.ddxt_ifc, nh, ldh);
+      t.ddxn_mc = up(ht.ddxn_mc, nf, ldf, p->cpd);
+      t.qdzh_c = up(ht.inv_dzh_c, nh, ldh, 0.5);
+      t.inv_dzm_c = up(ht.inv_dzm_c, nf, ldf);
+      t.fx_ratio = up(ht.fx_ratio, nf, ldf);
+      t.wcc0 = A.template alloc<T>(nc * ldh);
+      t.wcc1 = A.template alloc<T>(nc * ldh);
     };
     if (p->precision == ICON_PREC_FP64)
       build_terr(en.c64, double{});
@@ -806,7 +819,7 @@ int create_dycore(const icon_grid_t* grid, int nlev, const double* z_ifc, const 
   w.rho_p = A.alloc<double>(cf);
   w.theta_p = A.alloc<double>(cf);
   w.w_p = A.alloc<double>(ch);
-  w.pex = A.alloc<double>(cf);
+  w.pex = A.alloc<double>(is_mixed(p->precision) ? (size_t)nc * ld32 : cf);
   w.col = A.alloc<double>(8 * (cf + (size_t)kColWide * nlev));  // whole groups of columns
   w.diag = A.alloc<double>(diag_partials(nc));
   w.flag = A.alloc<int>(1);
@@ -1358,40 +1371,44 @@ int icon_profile_end(int32_t max_kernels, char* names, int32_t* launches, double
 int icon_dycore_debug_field(icon_dycore_t* d, const char* name, void* dst, int64_t bytes) {
   if (!d || !name || !dst) return fail(ICON_ERR_ARG, "icon_dycore_debug_field: NULL argument");
   const HostGrid& h = d->grid->host;
-  const size_t nlev = d->nlev, ef = h.ne * nlev, cf = h.nc * nlev, ch = h.nc * (nlev + 1);
+  const size_t nlev = d->nlev, nc = h.nc, ne = h.ne;
   const bool mixed = is_mixed(d->en.precision);
   const size_t es = mixed ? sizeof(float) : sizeof(double);
   const void* src = nullptr;
-  size_t n = 0;
-  auto pick = [&](const char* nm, const void* p64, const void* p32, size_t count, size_t elem) {
+  size_t n = 0, rows = 0, width = 0, pitch = 0;  // bytes but the rows
+  auto pick = [&](const char* nm, const void* p64, const void* p32, size_t n_rows, size_t nk, size_t elem) {
     if (std::strcmp(name, nm) == 0) {
       src = mixed ? p32 : p64;
-      n = count * elem;
+      rows = n_rows;
+      width = nk * elem;
+      n = rows * width;
+      // FP32 stencil fields have padded rows
+      pitch = elem == sizeof(float) ? d->en.c32.v.ldf * sizeof(float) : width;
     }
   };
   const WorkT<double>& a = d->en.c64.w;
   const WorkT<float>& b = d->en.c32.w;
-  pick("vt", a.vt, b.vt, ef, es);
-  pick("ekin_e", a.ekin_e, b.ekin_e, ef, es);
-  pick("ddt_vn0", a.ddt_vn0, b.ddt_vn0, ef, es);
-  pick("ddt_vn1", a.ddt_vn1, b.ddt_vn1, ef, es);
-  pick("rho_e", a.rho_e, b.rho_e, ef, es);
-  pick("theta_e", a.theta_e, b.theta_e, ef, es);
-  pick("hpg", a.hpg, b.hpg, ef, es);
-  pick("vn_p", a.vn_p, b.vn_p, ef, es);
-  pick("divd", a.divd, b.divd, cf, es);
-  pick("divd2", a.divd2, b.divd2, cf, es);
-  pick("ddt_w0", a.ddt_w0, b.ddt_w0, ch, es);
-  pick("ddt_w1", a.ddt_w1, b.ddt_w1, ch, es);
-  pick("grad4", a.grad4, b.grad4, 4 * cf, es);
-  pick("div_m", d->en.wk.div_m, d->en.wk.div_m, cf, sizeof(double));
-  pick("div_t", d->en.wk.div_t, d->en.wk.div_t, cf, sizeof(double));
-  pick("w_p", d->en.wk.w_p, d->en.m.w_p, ch, es);
-  pick("rho_p", d->en.wk.rho_p, d->en.wk.rho_p, cf, sizeof(double));
-  pick("theta_p", d->en.wk.theta_p, d->en.wk.theta_p, cf, sizeof(double));
+  pick("vt", a.vt, b.vt, ne, nlev, es);
+  pick("ekin_e", a.ekin_e, b.ekin_e, ne, nlev, es);
+  pick("ddt_vn0", a.ddt_vn0, b.ddt_vn0, ne, nlev, es);
+  pick("ddt_vn1", a.ddt_vn1, b.ddt_vn1, ne, nlev, es);
+  pick("rho_e", a.rho_e, b.rho_e, ne, nlev, es);
+  pick("theta_e", a.theta_e, b.theta_e, ne, nlev, es);
+  pick("hpg", a.hpg, b.hpg, ne, nlev, es);
+  pick("vn_p", a.vn_p, b.vn_p, ne, nlev, es);
+  pick("divd", a.divd, b.divd, nc, nlev, es);
+  pick("divd2", a.divd2, b.divd2, nc, nlev, es);
+  pick("ddt_w0", a.ddt_w0, b.ddt_w0, nc, nlev + 1, es);
+  pick("ddt_w1", a.ddt_w1, b.ddt_w1, nc, nlev + 1, es);
+  pick("grad4", a.grad4, b.grad4, 4 * nc, nlev, es);
+  pick("div_m", d->en.wk.div_m, d->en.wk.div_m, nc, nlev, sizeof(double));
+  pick("div_t", d->en.wk.div_t, d->en.wk.div_t, nc, nlev, sizeof(double));
+  pick("w_p", d->en.wk.w_p, d->en.m.w_p, nc, nlev + 1, es);
+  pick("rho_p", d->en.wk.rho_p, d->en.wk.rho_p, nc, nlev, sizeof(double));
+  pick("theta_p", d->en.wk.theta_p, d->en.wk.theta_p, nc, nlev, sizeof(double));
   if (!src) return fail(ICON_ERR_ARG, std::string("icon_dycore_debug_field: unknown field ") + name);
   if (bytes < (int64_t)n) return fail(ICON_ERR_ARG, "icon_dycore_debug_field: destination too small");
-  CUDA_TRY(cudaMemcpyAsync(dst, src, n, cudaMemcpyDeviceToDevice, d->stream));
+  CUDA_TRY(cudaMemcpy2DAsync(dst, width, src, pitch, width, rows, cudaMemcpyDeviceToDevice, d->stream));
   CUDA_TRY(cudaStreamSynchronize(d->stream));
   return ICON_OK;
 }

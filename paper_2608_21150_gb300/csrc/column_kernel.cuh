@@ -182,6 +182,8 @@ struct ColArgs {
   const double* rho_ref;
   // terrain: contravariant correction of the winds (cells, half levels)
   const T* wcc;
+  // row stride of the fields of type T and of the mirrors
+  int ldt;
 };
 
 // Arithmetic of the solve: FP64 (R = double), or double-word FP32 (R = dws,
@@ -427,31 +429,32 @@ __global__ void __launch_bounds__(ColForm<T, KC, CW, RL, kCorr != 0, kTerr>::NT,
   // levels k < n_ray may be Rayleigh-damped (the factor is 1 below)
   const int n_ray = v.n_ray;
 
-  // element offsets of worker wt's copies (full- and half-level fields)
-  auto offsets = [&](int wt, size_t* of, size_t* oh) {
+  // element offsets of worker wt's copies (FP64 full and half levels, type T)
+  auto offsets = [&](int wt, size_t* of, size_t* oh, size_t* ot) {
 #pragma unroll
     for (int j = 0; j < RL; ++j) {
       const int i = wt + j * F::NW;
       const size_t r = min(c0 + i / KC, nc - 1);
       of[j] = r * nlev + i % KC;
       oh[j] = r * nlevp + i % KC;
+      ot[j] = r * a.ldt + i % KC;
     }
   };
   const unsigned long long pol = policy_evict_last();
   auto load_chunk = [&](int k0, int wt) {
     const int nk = min(KC, nlev - k0);
-    size_t of[RL], oh[RL];
-    offsets(wt, of, oh);
+    size_t of[RL], oh[RL], ot[RL];
+    offsets(wt, of, oh, ot);
     tile_rows<F, KC>(T_w, a.w, wt, oh, k0, nk, pol);
     tile_rows<F, KC>(T_rho, a.rho, wt, of, k0, nk, pol);
     tile_rows<F, KC>(T_th, a.theta, wt, of, k0, nk, pol);
     tile_rows<F, KC>(T_pi, a.exner, wt, of, k0, nk, pol);
     tile_rows<F, KC>(T_dm, a.div_m, wt, of, k0, nk, pol);
     tile_rows<F, KC>(T_dt, a.div_t, wt, of, k0, nk, pol);
-    tile_rows<F, KC>(T_dw0, a.ddt_w0, wt, oh, k0 + 1, nk, pol);
-    if constexpr (kTerr) tile_rows<F, KC>(T_wc, a.wcc, wt, oh, k0 + 1, nk, pol);
+    tile_rows<F, KC>(T_dw0, a.ddt_w0, wt, ot, k0 + 1, nk, pol);
+    if constexpr (kTerr) tile_rows<F, KC>(T_wc, a.wcc, wt, ot, k0 + 1, nk, pol);
     if (kCT && corrector) {
-      tile_rows<F, KC>(T_dw1, a.ddt_w1, wt, oh, k0 + 1, nk, pol);
+      tile_rows<F, KC>(T_dw1, a.ddt_w1, wt, ot, k0 + 1, nk, pol);
       tile_rows<F, KC>(T_rp, a.rho_p, wt, of, k0, nk, pol);
       tile_rows<F, KC>(T_tp, a.theta_p, wt, of, k0, nk, pol);
     }
@@ -759,7 +762,7 @@ __global__ void __launch_bounds__(ColForm<T, KC, CW, RL, kCorr != 0, kTerr>::NT,
           const R thnew = levc<R, CZB, kStage, kTerr>(v, L_s, k, k0, c, nc) * A::mad(cvd_o_rd, prnew, y.eb) *
                           A::inv(y.zb * rnew);
           R wt = wd;
-          if constexpr (kTerr) wt = minus_corr(wd, -a.wcc[(size_t)c * nlevp + k]);  // w = w_con + wcc
+          if constexpr (kTerr) wt = minus_corr(wd, -a.wcc[(size_t)c * a.ldt + k]);  // w = w_con + wcc
           if (!(kMirror && !corrector)) O_w[o] = A::out(wt);
           if (kPairs && !corrector) {
             // the mixed predictor's rho and theta_v stay double-word pairs (read by the corrector)
@@ -782,17 +785,17 @@ __global__ void __launch_bounds__(ColForm<T, KC, CW, RL, kCorr != 0, kTerr>::NT,
         }
       }
       sync_workers<F>();
-      size_t of[RL], oh[RL];
-      offsets(wt, of, oh);
+      size_t of[RL], oh[RL], ot[RL];
+      offsets(wt, of, oh, ot);
       if (a.w_o) store_rows<F, KC>(O_w, a.w_o, wt, oh, k0, nk, ncol);
       store_rows<F, KC>(O_rho, a.rho_o, wt, of, k0, nk, ncol);
       if (a.exner_o) store_rows<F, KC>(O_pi, a.exner_o, wt, of, k0, nk, ncol);
       store_rows<F, KC>(O_th, a.theta_o, wt, of, k0, nk, ncol);
       if constexpr (kMirror) {
-        if (a.m_w) store_rows<F, KC>(Q_w, a.m_w, wt, oh, k0, nk, ncol);
+        if (a.m_w) store_rows<F, KC>(Q_w, a.m_w, wt, ot, k0, nk, ncol);
         if (a.m_rho) {
-          store_rows<F, KC>(Q_rho, a.m_rho, wt, of, k0, nk, ncol);
-          store_rows<F, KC>(Q_th, a.m_th, wt, of, k0, nk, ncol);
+          store_rows<F, KC>(Q_rho, a.m_rho, wt, ot, k0, nk, ncol);
+          store_rows<F, KC>(Q_th, a.m_th, wt, ot, k0, nk, ncol);
         }
       }
     }
@@ -800,9 +803,9 @@ __global__ void __launch_bounds__(ColForm<T, KC, CW, RL, kCorr != 0, kTerr>::NT,
   }
   if (active && threadIdx.x < CW) {
     // the ground: w_con = 0, so w = wcc there (0 over flat ground)
-    const T wg = kTerr ? a.wcc[(size_t)c * nlevp + nlev] : T(0);
+    const T wg = kTerr ? a.wcc[(size_t)c * a.ldt + nlev] : T(0);
     if (a.w_o) a.w_o[(size_t)c * nlevp + nlev] = (double)wg;
-    if (a.m_w) a.m_w[(size_t)c * nlevp + nlev] = (float)wg;
+    if (a.m_w) a.m_w[(size_t)c * a.ldt + nlev] = (float)wg;
   }
 }
 
@@ -829,6 +832,7 @@ ColArgs<T> col_args(const Engine& en, int corrector, const StateView& st, const 
   a.div_t = wk.div_t;
   a.col = wk.col;
   a.rho_ref = en.rho_ref64;
+  a.ldt = std::is_same<T, float>::value ? en.c32.v.ldh : en.c64.v.ldh;
   constexpr bool mixed = std::is_same<T, float>::value;
   if (corrector) {
     a.w_o = st.w;

@@ -65,6 +65,10 @@ using DevGrid = GridT<double>;
 template <class T>
 struct VertT {
   int nlev;
+  // row strides of the stencil fields at full and half levels.  FP64: nlev and
+  // nlev + 1.  FP32: both nlev + 1 rounded up to a multiple of four, so that
+  // every row starts on 16 bytes (the per-level arrays below are padded alike)
+  int ldf, ldh;
   const T* inv_dz;     // [nlev]
   const T* inv_dzh;    // [nlev+1]
   const T* qdz;        // [nlev] inv_dz / 4 (the vertical advection of vn: a mean of four w values)
@@ -78,7 +82,7 @@ struct VertT {
 // Terrain-following vertical coordinate (half-level heights per column): the
 // per-point metrics of the stencil kernels in the compute type T, all null
 // over flat ground.  Edge heights are the mean of the two cells'; slopes are
-// those of the coordinate surfaces.
+// those of the coordinate surfaces.  Rows have VertT's strides.
 template <class T>
 struct TerrT {
   const T* wgt_e;     // [ne*(nlev+1)] interpolation weight of level k-1 at edge half level k (0 at the ends)
@@ -208,7 +212,7 @@ struct VaPatchT {
   const float *own_w;  // [4] per cell: e2c_wd, 0
 };
 
-// Work arrays of the stencil kernels, compute type T.
+// Work arrays of the stencil kernels, compute type T, in rows of VertT's strides.
 template <class T>
 struct WorkT {
   // edges, full levels
@@ -235,7 +239,7 @@ struct DevWork {
   double *div_m, *div_t;                  // cells: flux divergences (FP64 sums; double-word pairs in mixed mode)
   double *rho_p, *theta_p;                // cells: predicted state (the corrector's time averages)
   double* w_p;                            // cells, half levels
-  double* pex;   // cells: extrapolated exner perturbation (FP64, or double-word pairs in mixed mode)
+  double* pex;   // cells: extrapolated exner perturbation (FP64, or double-word pairs in mixed mode, rows of VertT's stride)
   double* col;   // column solve scratch [level][group of columns][8 planes][column] (column_kernel.cuh)
   double* diag;  // diagnostics: partial column-mass sums
   int* flag;     // diagnostics: non-finite flag
@@ -243,7 +247,7 @@ struct DevWork {
 
 // FP32 mirrors of the state read by the mixed-mode stencils: vn, w, the
 // perturbations rho - rho_ref and theta_v - theta_ref, and the predicted w.
-// Written by the FP64 writers.
+// Written by the FP64 writers, in rows of VertT's strides.
 struct Mirrors {
   float *vn, *w, *rho, *th, *w_p;
 };

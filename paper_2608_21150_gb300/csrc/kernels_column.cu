@@ -315,6 +315,7 @@ extern "C" int icon_column_solve_noalloc(int32_t n_cols, int32_t nlev, const dou
   a.theta_p = theta_pred;
   a.div_m = div_m;
   a.div_t = div_t;
+  a.ldt = nlev + 1;
   a.col = base + kNoallocCoef;
   a.w_o = w_new;
   a.rho_o = rho_new;

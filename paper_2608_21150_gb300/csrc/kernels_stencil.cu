@@ -1,11 +1,12 @@
-// Stencil kernels of one dycore step (rows A1-A6, A8-A10), templated on the
-// compute type T: double (FP64 mode) or float (mixed mode, row A12).
+// Stencil kernels of one dycore step (rows A1-A6, A8-A10).  The FP64 kernels
+// stand here, with the edge kernels of the mixed modes that work a level at a
+// time (row A12); the other FP32 kernels, four levels per thread, are in
+// stencil_quad.cuh.
 //
-// Layout: level-contiguous X[h * nk + k] (k = 0 at the model top); one thread
-// per (horizontal point, level), flattened so that the 32 lanes of a warp
-// cover consecutive levels of one or two columns (the FP32 forms of five
-// gather-heavy kernels: one warp per point instead, see blocks_by_point).
-// Neighbour gathers X[nbr * nk + k] are coalesced runs of consecutive levels.
+// Layout: level-contiguous X[h * ld + k] (k = 0 at the model top).  FP64: one
+// thread per (horizontal point, level), flattened so that the 32 lanes of a
+// warp cover consecutive levels of one or two columns.  Neighbour gathers
+// X[nbr * ld + k] are coalesced runs of consecutive levels.
 //
 // Mixed mode: the stencils read FP32 mirrors of the state (vn, w and the
 // perturbations rho - rho_ref, theta_v - theta_ref) and compute in FP32,
@@ -18,6 +19,7 @@
 // operations, once per value by its writer, never per gather.
 #include <cuda_runtime.h>
 
+#include <initializer_list>
 #include <type_traits>
 
 #include "dfloat.cuh"
@@ -52,22 +54,16 @@ inline unsigned blocks_for(long long n, int threads) { return (unsigned)((n + th
 __device__ __forceinline__ double fmat(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float fmat(float a, float b, float c) { return fmaf(a, b, c); }
 
-// Second launch shape, used by the FP32 forms of the kernels whose per-point
-// gathers dominate (va_edge_pre, va_cell_w, sn_cell_div, sn_cell_fluxdiv,
-// sn_edge_corr): one warp per horizontal point, its lanes striding over the
-// levels, so the point's neighbour indices and weights are loaded once per
-// warp.  Not used for FP64, where 90 levels fill only 90 of 96 lane slots of
-// the saturated FP64 pipe, nor for the kernels that measured slower with it.
+// Second launch shape of va_edge_pre, va_cell_w, sn_cell_div and sn_edge_corr:
+// one warp per horizontal point, its lanes striding over the levels, so the
+// point's neighbour indices and weights are loaded once per warp.  The default
+// of the FP32 sn_edge_corr; not of the FP64 kernels, where 90 levels fill only
+// 90 of 96 lane slots of the saturated FP64 pipe (the tuner tries both).
 __device__ __forceinline__ int warp_point() { return (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); }
 __device__ __forceinline__ int lane_id() { return (int)(threadIdx.x & 31u); }
 inline unsigned blocks_for_points(long long n_points, int threads) {
   const int warps = threads / 32;
   return (unsigned)((n_points + warps - 1) / warps);
-}
-// CTAs of a kernel over n_h points and nk levels in the shape of its type
-template <class T>
-unsigned blocks_by_point(long long n_h, int nk, int threads) {
-  return kMixed<T> ? blocks_for_points(n_h, threads) : blocks_for(n_h * nk, threads);
 }
 // CTAs of a two-shape kernel: shape 1 one warp per point, 0 one thread per (point, level)
 inline unsigned blocks_by_shape(int shape, long long n_h, int nk, int threads) {
@@ -93,6 +89,12 @@ const char* kname(const char* f64, const char* f32) {
   return kMixed<T> ? f32 : f64;
 }
 
+}  // namespace
+}  // namespace icon
+#include "stencil_quad.cuh"
+namespace icon {
+namespace {
+
 // -------------------------------------------------------------------------
 // A1: tangential wind and edge kinetic energy
 //   vt = sum_j vt_w[j] vn[e_j] (Perot reconstruction averaged over the two
@@ -104,39 +106,39 @@ const char* kname(const char* f64, const char* f32) {
 // top and the lowest level's at the ground), for the edge tendency kernel.
 // Both tile shapes evaluate every (edge, level) with the same explicit FMAs
 // (va_edge_pre_at), so the autotuner's choice of shape does not change a bit.
-template <class T>
-__device__ __forceinline__ void va_edge_pre_at(const VertT<T>& v, int e, int k, int nlev, const T* x0, const T* x1,
-                                               const T* x2, const T* x3, const T* x4, const T* w, T* vt, T* ekin,
-                                               T* vn_ie, const T* wgt_e) {
+__device__ __forceinline__ void va_edge_pre_at(const VertT<double>& v, int e, int k, int nlev, const double* x0,
+                                               const double* x1, const double* x2, const double* x3, const double* x4,
+                                               const double* w, double* vt, double* ekin, double* vn_ie,
+                                               const double* wgt_e) {
   const int nlevp = nlev + 1;
-  const T vne = x0[k];
-  T t = w[0] * vne;
+  const double vne = x0[k];
+  double t = w[0] * vne;
   t = fmat(w[1], x1[k], t);
   t = fmat(w[2], x2[k], t);
   t = fmat(w[3], x3[k], t);
   t = fmat(w[4], x4[k], t);
   vt[(size_t)e * nlev + k] = t;
   ekin[(size_t)e * nlev + k] = fmat(vne, vne, t * t);
-  const T wg = wgt_e ? wgt_e[(size_t)e * nlevp + k] : v.wgt[k];
+  const double wg = wgt_e ? wgt_e[(size_t)e * nlevp + k] : v.wgt[k];
   vn_ie[(size_t)e * nlevp + k] = k == 0 ? vne : fmat(wg, x0[k - 1] - vne, vne);
   if (k == nlev - 1) vn_ie[(size_t)e * nlevp + nlev] = vne;
 }
 
-template <class T>
-__global__ void va_edge_pre(GridT<T> g, VertT<T> v, const T* __restrict__ vn, T* __restrict__ vt,
-                            T* __restrict__ ekin, T* __restrict__ vn_ie, const T* __restrict__ wgt_e, int shape) {
+__global__ void va_edge_pre(GridT<double> g, VertT<double> v, const double* __restrict__ vn, double* __restrict__ vt,
+                            double* __restrict__ ekin, double* __restrict__ vn_ie, const double* __restrict__ wgt_e,
+                            int shape) {
   const int nlev = v.nlev;
   if (shape) {  // one warp per edge, its lanes over the levels
     const int e = warp_point();
     if (e >= g.ne) return;
-    const T* w = g.vt_w + 5 * (size_t)e;
-    const T wl[5] = {w[0], w[1], w[2], w[3], w[4]};
+    const double* w = g.vt_w + 5 * (size_t)e;
+    const double wl[5] = {w[0], w[1], w[2], w[3], w[4]};
     const int* q = g.e2c2e + 4 * (size_t)e;
-    const T* x0 = vn + (size_t)e * nlev;
-    const T* x1 = vn + (size_t)q[0] * nlev;
-    const T* x2 = vn + (size_t)q[1] * nlev;
-    const T* x3 = vn + (size_t)q[2] * nlev;
-    const T* x4 = vn + (size_t)q[3] * nlev;
+    const double* x0 = vn + (size_t)e * nlev;
+    const double* x1 = vn + (size_t)q[0] * nlev;
+    const double* x2 = vn + (size_t)q[1] * nlev;
+    const double* x3 = vn + (size_t)q[2] * nlev;
+    const double* x4 = vn + (size_t)q[3] * nlev;
     for (int k = lane_id(); k < nlev; k += 32) va_edge_pre_at(v, e, k, nlev, x0, x1, x2, x3, x4, wl, vt, ekin, vn_ie, wgt_e);
     return;
   }
@@ -155,23 +157,22 @@ __global__ void va_edge_pre(GridT<T> g, VertT<T> v, const T* __restrict__ vn, T*
 // lowest full level's values at the ground; vn_ie from va_edge_pre; the
 // slopes vanish at the flat model top, where wcc = 0).
 // -------------------------------------------------------------------------
-template <class T>
-__global__ void va_concorr(GridT<T> g, VertT<T> v, TerrT<T> tr, const T* __restrict__ vn_ie,
-                           const T* __restrict__ vt, T* __restrict__ wcc) {
+__global__ void va_concorr(GridT<double> g, VertT<double> v, TerrT<double> tr, const double* __restrict__ vn_ie,
+                           const double* __restrict__ vt, double* __restrict__ wcc) {
   int c, k;
   const int nlev = v.nlev, nlevp = nlev + 1;
   if (!flat_index(g.nc, nlevp, c, k)) return;
-  T s = 0;
+  double s = 0;
   if (k > 0) {
     const int* ce = g.c2e + 3 * (size_t)c;
-    const T* q = g.e2c_w + 3 * (size_t)c;
+    const double* q = g.e2c_w + 3 * (size_t)c;
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
       const int e = ce[j];
-      const T* y = vt + (size_t)e * nlev;
+      const double* y = vt + (size_t)e * nlev;
       const size_t ih = (size_t)e * nlevp + k;
-      const T a = vn_ie[ih];
-      const T b = k == nlev ? y[nlev - 1] : y[k] + tr.wgt_e[ih] * (y[k - 1] - y[k]);
+      const double a = vn_ie[ih];
+      const double b = k == nlev ? y[nlev - 1] : y[k] + tr.wgt_e[ih] * (y[k - 1] - y[k]);
       s += q[j] * (a * tr.ddxn_ifc[ih] + b * tr.ddxt_ifc[ih]);
     }
   }
@@ -190,43 +191,36 @@ __global__ void va_concorr(GridT<T> g, VertT<T> v, TerrT<T> tr, const T* __restr
 // operations (the damping increment is a small part of vn, so the
 // cancellation in the sum costs nothing measurable); FP32 keeps the
 // differences.
-template <class T>
-__global__ void va_cell_vert(GridT<T> g, VertT<T> v, const T* __restrict__ vn, const T* __restrict__ w,
-                             const T* __restrict__ ekin_e, T* __restrict__ ekin_c, const T* __restrict__ divd,
-                             T* __restrict__ divd2, T* __restrict__ zeta, T* __restrict__ w_v, T* __restrict__ wq,
-                             const T* __restrict__ wcc) {
+__global__ void va_cell_vert(GridT<double> g, VertT<double> v, const double* __restrict__ vn,
+                             const double* __restrict__ w, const double* __restrict__ ekin_e,
+                             double* __restrict__ ekin_c, const double* __restrict__ divd, double* __restrict__ divd2,
+                             double* __restrict__ zeta, double* __restrict__ w_v, double* __restrict__ wq,
+                             const double* __restrict__ wcc) {
   const int nlev = v.nlev, nlevp = nlev + 1;
   unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
   const unsigned ncell = (unsigned)g.nc * nlev;
   if (i < ncell) {
     int c = (int)(i / (unsigned)nlev), k = (int)(i - (unsigned)c * nlev);
     const int* ce = g.c2e + 3 * (size_t)c;
-    const T* q = g.e2c_w + 3 * (size_t)c;
-    T s = q[0] * ekin_e[(size_t)ce[0] * nlev + k];
+    const double* q = g.e2c_w + 3 * (size_t)c;
+    double s = q[0] * ekin_e[(size_t)ce[0] * nlev + k];
     s += q[1] * ekin_e[(size_t)ce[1] * nlev + k];
     s += q[2] * ekin_e[(size_t)ce[2] * nlev + k];
     ekin_c[i] = s;
-    const T* wc = w + (size_t)c * nlevp;
+    const double* wc = w + (size_t)c * nlevp;
     if (wcc) {
-      const T* qc = wcc + (size_t)c * nlevp;
+      const double* qc = wcc + (size_t)c * nlevp;
       wq[i] = (wc[k] - qc[k]) + (wc[k + 1] - qc[k + 1]);
     } else {
       wq[i] = wc[k] + wc[k + 1];
     }
     if (divd2) {
       const int* cc = g.c2e2c + 3 * (size_t)c;
-      const T* L = g.lap_c + 3 * (size_t)c;
-      const T dc = divd[i];
-      const T d0 = divd[(size_t)cc[0] * nlev + k], d1 = divd[(size_t)cc[1] * nlev + k],
+      const double* L = g.lap_c + 3 * (size_t)c;
+      const double dc = divd[i];
+      const double d0 = divd[(size_t)cc[0] * nlev + k], d1 = divd[(size_t)cc[1] * nlev + k],
               d2 = divd[(size_t)cc[2] * nlev + k];
-      if constexpr (kMixed<T>) {
-        T r = L[0] * (d0 - dc);
-        r += L[1] * (d1 - dc);
-        r += L[2] * (d2 - dc);
-        divd2[i] = r;
-      } else {
-        divd2[i] = fmat(L[2], d2, fmat(L[1], d1, fmat(L[0], d0, -(g.lap_s[c] * dc))));
-      }
+      divd2[i] = fmat(L[2], d2, fmat(L[1], d1, fmat(L[0], d0, -(g.lap_s[c] * dc))));
     }
     return;
   }
@@ -235,15 +229,15 @@ __global__ void va_cell_vert(GridT<T> g, VertT<T> v, const T* __restrict__ vn, c
   int vx = (int)(i / (unsigned)nlevp), k = (int)(i - (unsigned)vx * nlevp);
   const int* ve = g.v2e + 6 * (size_t)vx;
   const int* vc = g.v2c + 6 * (size_t)vx;
-  const T* cw = g.curl_v + 6 * (size_t)vx;
-  const T* rw = g.c2v_w + 6 * (size_t)vx;
+  const double* cw = g.curl_v + 6 * (size_t)vx;
+  const double* rw = g.c2v_w + 6 * (size_t)vx;
   if (k < nlev) {
-    T z = 0;
+    double z = 0;
 #pragma unroll
     for (int j = 0; j < 6; ++j) z += cw[j] * vn[(size_t)ve[j] * nlev + k];
     zeta[(size_t)vx * nlev + k] = z;
   }
-  T s = 0;
+  double s = 0;
 #pragma unroll
   for (int j = 0; j < 6; ++j) s += rw[j] * w[(size_t)vc[j] * nlevp + k];
   w_v[i] = s;
@@ -263,34 +257,35 @@ __global__ void va_cell_vert(GridT<T> g, VertT<T> v, const T* __restrict__ vn, c
 // dz^-1/4 stored, the Coriolis term's 1/2 folded into a multiply-add, the
 // gradient of 2K times 1/(2 d) into the final multiply-add.  gw_e is stored
 // times d_e (its 1/d_e is folded into va_cell_w's weights).
-template <class T, bool kTerr = false>
-__global__ void va_edge_tend(GridT<T> g, VertT<T> v, const T* __restrict__ vn_ie, const T* __restrict__ w,
-                             const T* __restrict__ vt, const T* __restrict__ ekin_c, const T* __restrict__ zeta,
-                             const T* __restrict__ w_v, T* __restrict__ ddt_vn, T* __restrict__ gw_e, TerrT<T> tr,
-                             const T* __restrict__ wq) {
+template <bool kTerr = false>
+__global__ void va_edge_tend(GridT<double> g, VertT<double> v, const double* __restrict__ vn_ie,
+                             const double* __restrict__ w, const double* __restrict__ vt,
+                             const double* __restrict__ ekin_c, const double* __restrict__ zeta,
+                             const double* __restrict__ w_v, double* __restrict__ ddt_vn, double* __restrict__ gw_e,
+                             TerrT<double> tr, const double* __restrict__ wq) {
   int e, k;
   const int nlev = v.nlev, nlevp = nlev + 1;
   if (!flat_index(g.ne, nlevp, e, k)) return;
   const int c0 = g.e2c[2 * e], c1 = g.e2c[2 * e + 1];
-  const T* vte = vt + (size_t)e * nlev;
-  const T vnie_k = vn_ie[(size_t)e * nlevp + k];
+  const double* vte = vt + (size_t)e * nlev;
+  const double vnie_k = vn_ie[(size_t)e * nlevp + k];
   if (k < nlev) {
     const int vm = g.e2v[2 * e], vp = g.e2v[2 * e + 1];
-    const T vnie_k1 = vn_ie[(size_t)e * nlevp + k + 1];
-    const T ws = wq[(size_t)c0 * nlev + k] + wq[(size_t)c1 * nlev + k];
-    const T qdz = kTerr ? tr.qdz_e[(size_t)e * nlev + k] : v.qdz[k];
-    const T adv = (ws * (vnie_k - vnie_k1)) * qdz;
-    const T zf = fmat(T(0.5), zeta[(size_t)vm * nlev + k] + zeta[(size_t)vp * nlev + k], g.f_e[e]);
-    const T dk = ekin_c[(size_t)c0 * nlev + k] - ekin_c[(size_t)c1 * nlev + k];
+    const double vnie_k1 = vn_ie[(size_t)e * nlevp + k + 1];
+    const double ws = wq[(size_t)c0 * nlev + k] + wq[(size_t)c1 * nlev + k];
+    const double qdz = kTerr ? tr.qdz_e[(size_t)e * nlev + k] : v.qdz[k];
+    const double adv = (ws * (vnie_k - vnie_k1)) * qdz;
+    const double zf = fmat(double(0.5), zeta[(size_t)vm * nlev + k] + zeta[(size_t)vp * nlev + k], g.f_e[e]);
+    const double dk = ekin_c[(size_t)c0 * nlev + k] - ekin_c[(size_t)c1 * nlev + k];
     ddt_vn[(size_t)e * nlev + k] = fmat(dk, g.hinv_d[e], fmat(zf, vte[k], -adv));
   }
-  T gw = 0;
+  double gw = 0;
   if (k > 0 && k < nlev) {
     const int vm = g.e2v[2 * e], vp = g.e2v[2 * e + 1];
-    const T wg = kTerr ? tr.wgt_e[(size_t)e * nlevp + k] : v.wgt[k];
-    const T vtie = vte[k] + wg * (vte[k - 1] - vte[k]);
-    const T dwn = w[(size_t)c1 * nlevp + k] - w[(size_t)c0 * nlevp + k];
-    const T dwt = (w_v[(size_t)vp * nlevp + k] - w_v[(size_t)vm * nlevp + k]) * g.d_o_l[e];
+    const double wg = kTerr ? tr.wgt_e[(size_t)e * nlevp + k] : v.wgt[k];
+    const double vtie = vte[k] + wg * (vte[k - 1] - vte[k]);
+    const double dwn = w[(size_t)c1 * nlevp + k] - w[(size_t)c0 * nlevp + k];
+    const double dwt = (w_v[(size_t)vp * nlevp + k] - w_v[(size_t)vm * nlevp + k]) * g.d_o_l[e];
     gw = fmat(vnie_k, dwn, vtie * dwt);
   }
   gw_e[(size_t)e * nlevp + k] = gw;
@@ -303,15 +298,15 @@ __global__ void va_edge_tend(GridT<T> g, VertT<T> v, const T* __restrict__ vn_ie
 // -------------------------------------------------------------------------
 // Over terrain (kTerr): advected by w - wcc, per-cell half-level spacing.
 // Both tile shapes evaluate every (cell, half level) with va_cell_w_at.
-template <class T, bool kTerr>
-__device__ __forceinline__ T va_cell_w_at(const VertT<T>& v, const TerrT<T>& tr, int c, int k, int nlev,
-                                          const T* g0, const T* g1, const T* g2, const T* q, const T* wc,
-                                          const T* wcc) {
-  if (k == 0 || k >= nlev) return T(0);
-  const T h = fmat(q[2], g2[k], fmat(q[1], g1[k], q[0] * g0[k]));
+template <bool kTerr>
+__device__ __forceinline__ double va_cell_w_at(const VertT<double>& v, const TerrT<double>& tr, int c, int k, int nlev,
+                                               const double* g0, const double* g1, const double* g2, const double* q,
+                                               const double* wc, const double* wcc) {
+  if (k == 0 || k >= nlev) return double(0);
+  const double h = fmat(q[2], g2[k], fmat(q[1], g1[k], q[0] * g0[k]));
   // the difference of the full-level means above and below, (w_k-1 - w_k+1) / 2,
   // with the 1/2 folded into the stored 1/(2 dzh)
-  T wa, qd;
+  double wa, qd;
   if constexpr (kTerr) {
     const size_t ih = (size_t)c * (nlev + 1) + k;
     wa = wc[k] - wcc[ih];
@@ -323,29 +318,30 @@ __device__ __forceinline__ T va_cell_w_at(const VertT<T>& v, const TerrT<T>& tr,
   return fmat(-(wa * (wc[k - 1] - wc[k + 1])), qd, -h);
 }
 
-template <class T, bool kTerr = false>
-__global__ void va_cell_w(GridT<T> g, VertT<T> v, const T* __restrict__ w, const T* __restrict__ gw_e,
-                          T* __restrict__ ddt_w, TerrT<T> tr, const T* __restrict__ wcc, int shape) {
+template <bool kTerr = false>
+__global__ void va_cell_w(GridT<double> g, VertT<double> v, const double* __restrict__ w,
+                          const double* __restrict__ gw_e, double* __restrict__ ddt_w, TerrT<double> tr,
+                          const double* __restrict__ wcc, int shape) {
   const int nlev = v.nlev, nlevp = nlev + 1;
   if (shape) {  // one warp per cell, its lanes over the half levels
     const int c = warp_point();
     if (c >= g.nc) return;
     const int* ce = g.c2e + 3 * (size_t)c;
-    const T* qp = g.e2c_wd + 3 * (size_t)c;
-    const T q[3] = {qp[0], qp[1], qp[2]};
-    const T* g0 = gw_e + (size_t)ce[0] * nlevp;
-    const T* g1 = gw_e + (size_t)ce[1] * nlevp;
-    const T* g2 = gw_e + (size_t)ce[2] * nlevp;
-    const T* wc = w + (size_t)c * nlevp;
+    const double* qp = g.e2c_wd + 3 * (size_t)c;
+    const double q[3] = {qp[0], qp[1], qp[2]};
+    const double* g0 = gw_e + (size_t)ce[0] * nlevp;
+    const double* g1 = gw_e + (size_t)ce[1] * nlevp;
+    const double* g2 = gw_e + (size_t)ce[2] * nlevp;
+    const double* wc = w + (size_t)c * nlevp;
     for (int k = lane_id(); k < nlevp; k += 32)
-      ddt_w[(size_t)c * nlevp + k] = va_cell_w_at<T, kTerr>(v, tr, c, k, nlev, g0, g1, g2, q, wc, wcc);
+      ddt_w[(size_t)c * nlevp + k] = va_cell_w_at<kTerr>(v, tr, c, k, nlev, g0, g1, g2, q, wc, wcc);
     return;
   }
   int c, k;
   if (!flat_index(g.nc, nlevp, c, k)) return;
   const int* ce = g.c2e + 3 * (size_t)c;
   ddt_w[(size_t)c * nlevp + k] =
-      va_cell_w_at<T, kTerr>(v, tr, c, k, nlev, gw_e + (size_t)ce[0] * nlevp, gw_e + (size_t)ce[1] * nlevp,
+      va_cell_w_at<kTerr>(v, tr, c, k, nlev, gw_e + (size_t)ce[0] * nlevp, gw_e + (size_t)ce[1] * nlevp,
                              gw_e + (size_t)ce[2] * nlevp, g.e2c_wd + 3 * (size_t)c, w + (size_t)c * nlevp, wcc);
 }
 
@@ -397,7 +393,7 @@ __global__ void __launch_bounds__(kVaThreads, 2) va_fused(GridT<float> g, VertT<
   extern __shared__ float sf[];
   constexpr int L = kVaL, S = kVaS, Sn = kVaSn;
   const int p = blockIdx.x;
-  const int nlev = v.nlev, nlevp = nlev + 1;
+  const int nlev = v.nlev, ld = v.ldf;
   const int e0a = pt.off_e0[p], ne0 = pt.off_e0[p + 1] - e0a;
   const int e1a = pt.off_e1[p], ne1 = pt.off_e1[p + 1] - e1a;
   const int c0a = pt.off_c0[p], nc0 = pt.off_c0[p + 1] - c0a, nc3 = pt.n_c3[p];
@@ -423,11 +419,11 @@ __global__ void __launch_bounds__(kVaThreads, 2) va_fused(GridT<float> g, VertT<
       const int it = i / (L + 2), lv = i - it * (L + 2);
       if (it < ne0) {
         const int k = min(max(kc - 1 + lv, 0), nlev - 1);
-        cp_async4(vs + it * Sn + lv, vn + (size_t)pt.e0_g[e0a + it] * nlev + k);
+        cp_async4(vs + it * Sn + lv, vn + (size_t)pt.e0_g[e0a + it] * ld + k);
       } else {
         const int kh = min(max(kc - 1 + lv, 0), nlev);
         const int ic = it - ne0;
-        cp_async4(ws + ic * Sn + lv, w + (size_t)pt.c0_g[c0a + ic] * nlevp + kh);
+        cp_async4(ws + ic * Sn + lv, w + (size_t)pt.c0_g[c0a + ic] * ld + kh);
       }
     }
     cp_commit();
@@ -440,7 +436,7 @@ __global__ void __launch_bounds__(kVaThreads, 2) va_fused(GridT<float> g, VertT<
       const int kp = k0 - L;
       for (int i = threadIdx.x; i < ncown * L; i += blockDim.x) {
         const int it = i / L, lv = i - it * L, k = kp + lv;
-        if (k <= nlev) ddt_w[(size_t)(c_begin + it) * nlevp + k] = dw_s[it * S + lv];
+        if (k <= nlev) ddt_w[(size_t)(c_begin + it) * ld + k] = dw_s[it * S + lv];
       }
     }
     if (k0 > nlev) break;
@@ -495,7 +491,7 @@ __global__ void __launch_bounds__(kVaThreads, 2) va_fused(GridT<float> g, VertT<
     __syncthreads();
     for (int i = threadIdx.x; i < nw4 * L; i += blockDim.x) {  // vt of the edges this patch writes
       const int it = i / L, lv = i - it * L, k = k0 + lv;
-      if (k < nlev) vt_out[(size_t)pt.e4_g[e4a + it] * nlev + k] = vt_s[(int)pt.e4_i[8 * (size_t)(e4a + it)] * S + lv + 1];
+      if (k < nlev) vt_out[(size_t)pt.e4_g[e4a + it] * ld + k] = vt_s[(int)pt.e4_i[8 * (size_t)(e4a + it)] * S + lv + 1];
     }
     if (divd2) {  // the corrector's divergence-damping Laplacian at the own cells
       for (int i = threadIdx.x; i < ncown * L; i += blockDim.x) {
@@ -504,10 +500,10 @@ __global__ void __launch_bounds__(kVaThreads, 2) va_fused(GridT<float> g, VertT<
         const int c = c_begin + it;
         const int* cc = g.c2e2c + 3 * (size_t)c;
         const float* Lw = g.lap_c + 3 * (size_t)c;
-        const size_t ic = (size_t)c * nlev + k;
+        const size_t ic = (size_t)c * ld + k;
         const float dc = divd[ic];
-        const float d0 = divd[(size_t)cc[0] * nlev + k], d1 = divd[(size_t)cc[1] * nlev + k],
-                    d2 = divd[(size_t)cc[2] * nlev + k];
+        const float d0 = divd[(size_t)cc[0] * ld + k], d1 = divd[(size_t)cc[1] * ld + k],
+                    d2 = divd[(size_t)cc[2] * ld + k];
         float r = Lw[0] * (d0 - dc);
         r += Lw[1] * (d1 - dc);
         r += Lw[2] * (d2 - dc);
@@ -634,7 +630,7 @@ __global__ void __launch_bounds__(kVaThreads, 2) va_fused(GridT<float> g, VertT<
     }
     for (int i = threadIdx.x; i < nw4 * L; i += blockDim.x) {
       const int it = i / L, lv = i - it * L, k = k0 + lv;
-      if (k < nlev) ddt_vn[(size_t)pt.e4_g[e4a + it] * nlev + k] = dv_s[it * S + lv];
+      if (k < nlev) ddt_vn[(size_t)pt.e4_g[e4a + it] * ld + k] = dv_s[it * S + lv];
     }
   }
 }
@@ -645,50 +641,36 @@ __global__ void __launch_bounds__(kVaThreads, 2) va_fused(GridT<float> g, VertT<
 // frame: grad4 = (drho_x, drho_y, dth_x, dth_y) as 4 planes [4][nc*nlev].
 // -------------------------------------------------------------------------
 // exner_ref_c: the per-column reference exner over terrain (kTerr).
-template <class T, bool kTerr = false>
-__global__ void sn_cell_grad(GridT<T> g, VertT<T> v, const T* __restrict__ rho, const T* __restrict__ theta,
-                             T* __restrict__ grad4, const double* __restrict__ exner,
-                             const double* __restrict__ exner_pr, double exfac, double* __restrict__ pex,
-                             const double* __restrict__ exner_ref_c) {
+template <bool kTerr = false>
+__global__ void sn_cell_grad(GridT<double> g, VertT<double> v, const double* __restrict__ rho,
+                             const double* __restrict__ theta, double* __restrict__ grad4,
+                             const double* __restrict__ exner, const double* __restrict__ exner_pr, double exfac,
+                             double* __restrict__ pex, const double* __restrict__ exner_ref_c) {
   int c, k;
   const int nlev = v.nlev;
   if (!flat_index(g.nc, nlev, c, k)) return;
   const size_t n = (size_t)g.nc * nlev;
   const int* cc = g.c2e2c + 3 * (size_t)c;
-  const T* G = g.grad_c + 6 * (size_t)c;
+  const double* G = g.grad_c + 6 * (size_t)c;
   const size_t i = (size_t)c * nlev + k;
   const double ex_ref = kTerr ? exner_ref_c[i] : v.exner_ref[k];
   // extrapolated exner perturbation (1 + a) pr - a pr_old of this cell, for the
   // pressure gradient at its edges: FP64, or a double-word pair in mixed mode
   // (exner is near 1, the difference across an edge ~1e-5 of it)
-  if constexpr (kMixed<T>) {
-    const df a = to_df(1.0 + exfac), b = to_df(exfac);
-    reinterpret_cast<df*>(pex)[i] = a * (to_df(exner[i]) - to_df(ex_ref)) - b * to_df(exner_pr[i]);
-  } else {
-    pex[i] = (1.0 + exfac) * (exner[i] - ex_ref) - exfac * exner_pr[i];
-  }
+  pex[i] = (1.0 + exfac) * (exner[i] - ex_ref) - exfac * exner_pr[i];
   const size_t i0 = (size_t)cc[0] * nlev + k, i1 = (size_t)cc[1] * nlev + k, i2 = (size_t)cc[2] * nlev + k;
-  const T r = rho[i], t = theta[i];
-  if constexpr (kMixed<T>) {
-    const T r0 = rho[i0] - r, r1 = rho[i1] - r, r2 = rho[i2] - r;
-    const T t0 = theta[i0] - t, t1 = theta[i1] - t, t2 = theta[i2] - t;
-    grad4[i] = G[0] * r0 + G[2] * r1 + G[4] * r2;
-    grad4[n + i] = G[1] * r0 + G[3] * r1 + G[5] * r2;
-    grad4[2 * n + i] = G[0] * t0 + G[2] * t1 + G[4] * t2;
-    grad4[3 * n + i] = G[1] * t0 + G[3] * t1 + G[5] * t2;
-  } else {
-    // sum G_j psi_j - (sum G_j) psi_c: four FP64 operations per component
-    // instead of the differences' shared three plus three (the gradient only
-    // moves the upwind value by a small fraction of it, so the cancellation
-    // is harmless)
-    const T* S = g.grad_s + 2 * (size_t)c;
-    const T r0 = rho[i0], r1 = rho[i1], r2 = rho[i2];
-    const T t0 = theta[i0], t1 = theta[i1], t2 = theta[i2];
-    grad4[i] = fmat(G[4], r2, fmat(G[2], r1, fmat(G[0], r0, -(S[0] * r))));
-    grad4[n + i] = fmat(G[5], r2, fmat(G[3], r1, fmat(G[1], r0, -(S[1] * r))));
-    grad4[2 * n + i] = fmat(G[4], t2, fmat(G[2], t1, fmat(G[0], t0, -(S[0] * t))));
-    grad4[3 * n + i] = fmat(G[5], t2, fmat(G[3], t1, fmat(G[1], t0, -(S[1] * t))));
-  }
+  const double r = rho[i], t = theta[i];
+  // sum G_j psi_j - (sum G_j) psi_c: four FP64 operations per component
+  // instead of the differences' shared three plus three (the gradient only
+  // moves the upwind value by a small fraction of it, so the cancellation
+  // is harmless)
+  const double* S = g.grad_s + 2 * (size_t)c;
+  const double r0 = rho[i0], r1 = rho[i1], r2 = rho[i2];
+  const double t0 = theta[i0], t1 = theta[i1], t2 = theta[i2];
+  grad4[i] = fmat(G[4], r2, fmat(G[2], r1, fmat(G[0], r0, -(S[0] * r))));
+  grad4[n + i] = fmat(G[5], r2, fmat(G[3], r1, fmat(G[1], r0, -(S[1] * r))));
+  grad4[2 * n + i] = fmat(G[4], t2, fmat(G[2], t1, fmat(G[0], t0, -(S[0] * t))));
+  grad4[3 * n + i] = fmat(G[5], t2, fmat(G[3], t1, fmat(G[1], t0, -(S[1] * t))));
 }
 
 // -------------------------------------------------------------------------
@@ -704,59 +686,43 @@ __global__ void sn_cell_grad(GridT<T> g, VertT<T> v, const T* __restrict__ rho, 
 // horizontal: the along-level difference minus the slope of the full level
 // times the edge mean of the two cells' vertical derivatives (centred, one-
 // sided at the top and the ground) of the extrapolated exner perturbation.
-template <class T, bool kTerr = false>
-__global__ void sn_edge_pred(GridT<T> g, VertT<T> v, ScalT<T> sc, const T* __restrict__ vn,
-                             const T* __restrict__ vt, const T* __restrict__ ddt_vn, const T* __restrict__ rho,
-                             const T* __restrict__ theta, const double* __restrict__ pex,
-                             const double* __restrict__ cid64, const T* __restrict__ grad4, T* __restrict__ rho_e,
-                             T* __restrict__ theta_e,
-                             T* __restrict__ hpg, T* __restrict__ vn_p, TerrT<T> tr) {
+template <bool kTerr = false>
+__global__ void sn_edge_pred(GridT<double> g, VertT<double> v, ScalT<double> sc, const double* __restrict__ vn,
+                             const double* __restrict__ vt, const double* __restrict__ ddt_vn,
+                             const double* __restrict__ rho, const double* __restrict__ theta,
+                             const double* __restrict__ pex, const double* __restrict__ cid64,
+                             const double* __restrict__ grad4, double* __restrict__ rho_e, double* __restrict__ theta_e,
+                             double* __restrict__ hpg, double* __restrict__ vn_p, TerrT<double> tr) {
   int e, k;
   const int nlev = v.nlev;
   if (!flat_index(g.ne, nlev, e, k)) return;
   const size_t n = (size_t)g.nc * nlev;
   const size_t ie = (size_t)e * nlev + k;
-  const T vne = vn[ie], vte = vt[ie];
-  const int side = vne >= T(0) ? 0 : 1;
+  const double vne = vn[ie], vte = vt[ie];
+  const int side = vne >= double(0) ? 0 : 1;
   const int cu = g.e2c[2 * e + side];
   // offset of the back-trajectory point from the upwind cell's centre, with
   // the half substep folded into the stored normal and tangent: two FMAs each
-  const T* u = g.upw_s + 12 * (size_t)e + 6 * side;
-  const T dx = fmat(-vne, u[2], fmat(-vte, u[4], u[0]));
-  const T dy = fmat(-vne, u[3], fmat(-vte, u[5], u[1]));
+  const double* u = g.upw_s + 12 * (size_t)e + 6 * side;
+  const double dx = fmat(-vne, u[2], fmat(-vte, u[4], u[0]));
+  const double dy = fmat(-vne, u[3], fmat(-vte, u[5], u[1]));
   const size_t iu = (size_t)cu * nlev + k;
-  T ru = rho[iu], tu = theta[iu];
-  if constexpr (kMixed<T>) {
-    ru += v.rho_ref[k];
-    tu += v.theta_ref[k];
-  }
-  const T re = fmat(grad4[iu], dx, fmat(grad4[n + iu], dy, ru));
-  const T te = fmat(grad4[2 * n + iu], dx, fmat(grad4[3 * n + iu], dy, tu));
+  double ru = rho[iu], tu = theta[iu];
+  const double re = fmat(grad4[iu], dx, fmat(grad4[n + iu], dy, ru));
+  const double te = fmat(grad4[2 * n + iu], dx, fmat(grad4[3 * n + iu], dy, tu));
   const int c0 = g.e2c[2 * e], c1 = g.e2c[2 * e + 1];
   const size_t i0 = (size_t)c0 * nlev + k, i1 = (size_t)c1 * nlev + k;
   // cpd theta_e d(pr)/dn with cpd folded into the edge factor cpd / d_e (and,
   // over terrain, into the stored slope)
-  T h;
+  double h;
   const int km = k > 0 ? k - 1 : 0, kp = k + 1 < nlev ? k + 1 : nlev - 1;
-  if constexpr (kMixed<T>) {
-    const df* p = reinterpret_cast<const df*>(pex);
-    if constexpr (kTerr) {
-      const size_t b0 = (size_t)c0 * nlev, b1 = (size_t)c1 * nlev;
-      const T dz0 = to_float(p[b0 + km] - p[b0 + kp]) * tr.inv_dzm_c[i0];
-      const T dz1 = to_float(p[b1 + km] - p[b1 + kp]) * tr.inv_dzm_c[i1];
-      h = te * (to_float(p[i1] - p[i0]) * g.cpd_inv_d[e] - tr.ddxn_mc[ie] * (T(0.5) * (dz0 + dz1)));
-    } else {
-      h = te * (to_float(p[i1] - p[i0]) * g.cpd_inv_d[e]);
-    }
+  if constexpr (kTerr) {
+    const size_t b0 = (size_t)c0 * nlev, b1 = (size_t)c1 * nlev;
+    const double dz0 = (pex[b0 + km] - pex[b0 + kp]) * tr.inv_dzm_c[i0];
+    const double dz1 = (pex[b1 + km] - pex[b1 + kp]) * tr.inv_dzm_c[i1];
+    h = te * ((pex[i1] - pex[i0]) * cid64[e] - tr.ddxn_mc[ie] * (0.5 * (dz0 + dz1)));
   } else {
-    if constexpr (kTerr) {
-      const size_t b0 = (size_t)c0 * nlev, b1 = (size_t)c1 * nlev;
-      const double dz0 = (pex[b0 + km] - pex[b0 + kp]) * tr.inv_dzm_c[i0];
-      const double dz1 = (pex[b1 + km] - pex[b1 + kp]) * tr.inv_dzm_c[i1];
-      h = te * (T)((pex[i1] - pex[i0]) * cid64[e] - tr.ddxn_mc[ie] * (0.5 * (dz0 + dz1)));
-    } else {
-      h = te * (T)((pex[i1] - pex[i0]) * cid64[e]);
-    }
+    h = te * ((pex[i1] - pex[i0]) * cid64[e]);
   }
   rho_e[ie] = re;
   theta_e[ie] = te;
@@ -779,28 +745,30 @@ __global__ void sn_edge_hpg_steep(GridT<T> g, VertT<T> v, ScalT<T> sc, int n, co
                                   const T* __restrict__ ddt_vn, T* __restrict__ hpg, T* __restrict__ vn_p) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const int nlev = v.nlev;
+  const int nlev = v.nlev, ldf = v.ldf;
   const int e = idx[4 * i], k = idx[4 * i + 1];
   const int c0 = g.e2c[2 * e], c1 = g.e2c[2 * e + 1];
-  const size_t b0 = (size_t)c0 * nlev + idx[4 * i + 2], b1 = (size_t)c1 * nlev + idx[4 * i + 3];
+  const int l0 = idx[4 * i + 2], l1 = idx[4 * i + 3];
+  const size_t b0 = (size_t)c0 * ldf + l0, b1 = (size_t)c1 * ldf + l1;
+  const size_t r0 = (size_t)c0 * nlev + l0, r1 = (size_t)c1 * nlev + l1;
   const double* w = wts + 6 * (size_t)i;
-  const size_t ie = (size_t)e * nlev + k;
+  const size_t ie = (size_t)e * ldf + k;
   T h;
   if constexpr (kMixed<T>) {
     const df* p = reinterpret_cast<const df*>(pex);
     df s0{0.f, 0.f}, s1{0.f, 0.f};
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-      s0 = s0 + to_df(w[j]) * (p[b0 + j] + to_df(exref_c[b0 + j]));
-      s1 = s1 + to_df(w[3 + j]) * (p[b1 + j] + to_df(exref_c[b1 + j]));
+      s0 = s0 + to_df(w[j]) * (p[b0 + j] + to_df(exref_c[r0 + j]));
+      s1 = s1 + to_df(w[3 + j]) * (p[b1 + j] + to_df(exref_c[r1 + j]));
     }
     h = theta_e[ie] * (to_float(s1 - s0) * g.cpd_inv_d[e]);
   } else {
     double s0 = 0.0, s1 = 0.0;
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-      s0 = fma(w[j], pex[b0 + j] + exref_c[b0 + j], s0);
-      s1 = fma(w[3 + j], pex[b1 + j] + exref_c[b1 + j], s1);
+      s0 = fma(w[j], pex[b0 + j] + exref_c[r0 + j], s0);
+      s1 = fma(w[3 + j], pex[b1 + j] + exref_c[r1 + j], s1);
     }
     h = theta_e[ie] * (T)((s1 - s0) * cid64[e]);
   }
@@ -815,7 +783,7 @@ __global__ void sn_edge_hpg_steep(GridT<T> g, VertT<T> v, ScalT<T> sc, int n, co
 // -------------------------------------------------------------------------
 // Both tile shapes update every (edge, level) with sn_edge_corr_at.
 template <class T>
-__device__ __forceinline__ void sn_edge_corr_at(const ScalT<T>& sc, size_t ie, T ddamp, T d0k, T d1k,
+__device__ __forceinline__ void sn_edge_corr_at(const ScalT<T>& sc, size_t iv, size_t ie, T ddamp, T d0k, T d1k,
                                                 double* vn, const T* ddt_vn0, const T* ddt_vn1, const T* hpg,
                                                 float* m_vn) {
   // fourth-order divergence damping: divdamp_fac Abar^2 grad_n(dd2), coefficient per edge
@@ -823,11 +791,11 @@ __device__ __forceinline__ void sn_edge_corr_at(const ScalT<T>& sc, size_t ie, T
   const T tend = fmat(sc.wnow_vel, ddt_vn0[ie], fmat(sc.wnew_vel, ddt_vn1[ie], -hpg[ie]));
   const T inc = fmat(sc.dt_s, tend, -damp);
   if constexpr (kMixed<T>) {
-    const double vnn = vn[ie] + f2d(inc);
-    vn[ie] = vnn;
+    const double vnn = vn[iv] + f2d(inc);
+    vn[iv] = vnn;
     m_vn[ie] = d2f(vnn);
   } else {
-    vn[ie] = vn[ie] + (double)inc;
+    vn[iv] = vn[iv] + (double)inc;
   }
 }
 
@@ -836,23 +804,23 @@ __global__ void sn_edge_corr(GridT<T> g, VertT<T> v, ScalT<T> sc, double* __rest
                              const T* __restrict__ ddt_vn0, const T* __restrict__ ddt_vn1,
                              const T* __restrict__ hpg, const T* __restrict__ divd2, float* __restrict__ m_vn,
                              int shape) {
-  const int nlev = v.nlev;
+  const int nlev = v.nlev, ldf = v.ldf;
   if (shape) {  // one warp per edge, its lanes over the levels
     const int e = warp_point();
     if (e >= g.ne) return;
     const int c0 = g.e2c[2 * e], c1 = g.e2c[2 * e + 1];
     const T ddamp = g.ddamp_e[e];
-    const T* d0 = divd2 + (size_t)c0 * nlev;
-    const T* d1 = divd2 + (size_t)c1 * nlev;
+    const T* d0 = divd2 + (size_t)c0 * ldf;
+    const T* d1 = divd2 + (size_t)c1 * ldf;
     for (int k = lane_id(); k < nlev; k += 32)
-      sn_edge_corr_at(sc, (size_t)e * nlev + k, ddamp, d0[k], d1[k], vn, ddt_vn0, ddt_vn1, hpg, m_vn);
+      sn_edge_corr_at(sc, (size_t)e * nlev + k, (size_t)e * ldf + k, ddamp, d0[k], d1[k], vn, ddt_vn0, ddt_vn1, hpg, m_vn);
     return;
   }
   int e, k;
   if (!flat_index(g.ne, nlev, e, k)) return;
   const int c0 = g.e2c[2 * e], c1 = g.e2c[2 * e + 1];
-  sn_edge_corr_at(sc, (size_t)e * nlev + k, g.ddamp_e[e], divd2[(size_t)c0 * nlev + k],
-                  divd2[(size_t)c1 * nlev + k], vn, ddt_vn0, ddt_vn1, hpg, m_vn);
+  sn_edge_corr_at(sc, (size_t)e * nlev + k, (size_t)e * ldf + k, g.ddamp_e[e], divd2[(size_t)c0 * ldf + k],
+                  divd2[(size_t)c1 * ldf + k], vn, ddt_vn0, ddt_vn1, hpg, m_vn);
 }
 
 // -------------------------------------------------------------------------
@@ -862,8 +830,8 @@ __global__ void sn_edge_corr(GridT<T> g, VertT<T> v, ScalT<T> sc, double* __rest
 // exner_pr = exner - exner_ref (sn_edge_pred, its last reader, has completed).
 // Both tile shapes evaluate every (cell, level) with the same FMAs.
 // -------------------------------------------------------------------------
-template <class T, bool kTerr = false>
-__global__ void sn_cell_div(GridT<T> g, VertT<T> v, const T* __restrict__ vn, T* __restrict__ divd,
+template <bool kTerr = false>
+__global__ void sn_cell_div(GridT<double> g, VertT<double> v, const double* __restrict__ vn, double* __restrict__ divd,
                             const double* __restrict__ exner, double* __restrict__ exner_pr,
                             const double* __restrict__ exner_ref_c, int shape) {
   const int nlev = v.nlev;
@@ -871,11 +839,11 @@ __global__ void sn_cell_div(GridT<T> g, VertT<T> v, const T* __restrict__ vn, T*
     const int c = warp_point();
     if (c >= g.nc) return;
     const int* ce = g.c2e + 3 * (size_t)c;
-    const T* dvp = g.div_c + 3 * (size_t)c;
-    const T dv0 = dvp[0], dv1 = dvp[1], dv2 = dvp[2];
-    const T* x0 = vn + (size_t)ce[0] * nlev;
-    const T* x1 = vn + (size_t)ce[1] * nlev;
-    const T* x2 = vn + (size_t)ce[2] * nlev;
+    const double* dvp = g.div_c + 3 * (size_t)c;
+    const double dv0 = dvp[0], dv1 = dvp[1], dv2 = dvp[2];
+    const double* x0 = vn + (size_t)ce[0] * nlev;
+    const double* x1 = vn + (size_t)ce[1] * nlev;
+    const double* x2 = vn + (size_t)ce[2] * nlev;
     for (int k = lane_id(); k < nlev; k += 32) {
       const size_t i = (size_t)c * nlev + k;
       divd[i] = fmat(dv2, x2[k], fmat(dv1, x1[k], dv0 * x0[k]));
@@ -886,87 +854,11 @@ __global__ void sn_cell_div(GridT<T> g, VertT<T> v, const T* __restrict__ vn, T*
   int c, k;
   if (!flat_index(g.nc, nlev, c, k)) return;
   const int* ce = g.c2e + 3 * (size_t)c;
-  const T* dv = g.div_c + 3 * (size_t)c;
+  const double* dv = g.div_c + 3 * (size_t)c;
   const size_t i = (size_t)c * nlev + k;
   divd[i] = fmat(dv[2], vn[(size_t)ce[2] * nlev + k], fmat(dv[1], vn[(size_t)ce[1] * nlev + k],
                                                            dv[0] * vn[(size_t)ce[0] * nlev + k]));
   if (exner_pr) exner_pr[i] = exner[i] - (kTerr ? exner_ref_c[i] : v.exner_ref[k]);
-}
-
-// -------------------------------------------------------------------------
-// Divergences of the horizontal mass and theta fluxes with the flux-velocity
-// filter, per cell and level, summed in FP64 (double-word FP32 in mixed
-// mode, stored as the pair):
-//   vf_e = vn_e + divflux (D_c1 - D_c0)/d_e,  F_e = rho_e vf_e,
-//   div_m = sum s l F / A,  div_t = sum s l F theta_e / A
-// -------------------------------------------------------------------------
-// Over terrain (kTerr) each flux carries its edge layer thickness over the
-// cell's, fx_ratio = dz_e / dz_c: div_m = (1/dz_c) sum s l F dz_e / A.
-template <class T, bool kTerr = false>
-__global__ void sn_cell_fluxdiv(GridT<T> g, VertT<T> v, ScalT<T> sc, const T* __restrict__ vn,
-                                const T* __restrict__ divd, const T* __restrict__ rho_e,
-                                const T* __restrict__ theta_e, const double* __restrict__ div_c64,
-                                double* __restrict__ div_m, double* __restrict__ div_t,
-                                const T* __restrict__ fx_ratio) {
-  const int nlev = v.nlev;
-  if constexpr (kMixed<T>) {
-    // FP32 fluxes, sums in double-word FP32: FP64-grade accumulation (mass
-    // conserved to about 2^-48 of the flux) without the slow FP64 pipe.  One
-    // warp per cell: the cell's three edges, their filter coefficients and
-    // the divergence rows of their cells are loaded once.
-    const int c = warp_point();
-    if (c >= g.nc) return;
-    const int* ce = g.c2e + 3 * (size_t)c;
-    size_t be[3], bd0[3], bd1[3];
-    T fd[3];
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      const int e = ce[j];
-      be[j] = (size_t)e * nlev;
-      bd0[j] = (size_t)g.e2c[2 * e] * nlev;
-      bd1[j] = (size_t)g.e2c[2 * e + 1] * nlev;
-      fd[j] = g.fdiv_e[e];
-    }
-    const df* dvp = reinterpret_cast<const df*>(g.div_c_hl) + 3 * (size_t)c;
-    const df dv[3] = {dvp[0], dvp[1], dvp[2]};
-    for (int k = lane_id(); k < nlev; k += 32) {
-      df dm{0.f, 0.f}, dt{0.f, 0.f};
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        const size_t ie = be[j] + k;
-        const T vf = vn[ie] + fd[j] * (divd[bd1[j] + k] - divd[bd0[j] + k]);
-        T f = rho_e[ie] * vf;
-        if constexpr (kTerr) f = f * fx_ratio[((size_t)c * 3 + j) * nlev + k];
-        const T ft = f * theta_e[ie];
-        const df w = dv[j];
-        dm = dm + w * f;
-        dt = dt + w * ft;
-      }
-      // stored as the double-word pair itself (8 bytes, read by the column solve)
-      reinterpret_cast<df*>(div_m)[(size_t)c * nlev + k] = dm;
-      reinterpret_cast<df*>(div_t)[(size_t)c * nlev + k] = dt;
-    }
-  } else {
-    int c, k;
-    if (!flat_index(g.nc, nlev, c, k)) return;
-    const int* ce = g.c2e + 3 * (size_t)c;
-    const double* dv = div_c64 + 3 * (size_t)c;
-    double dm = 0.0, dt = 0.0;
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      const int e = ce[j];
-      const size_t ie = (size_t)e * nlev + k;
-      const int c0 = g.e2c[2 * e], c1 = g.e2c[2 * e + 1];
-      const T vf = vn[ie] + g.fdiv_e[e] * (divd[(size_t)c1 * nlev + k] - divd[(size_t)c0 * nlev + k]);
-      T f = rho_e[ie] * vf;
-      if constexpr (kTerr) f = f * fx_ratio[((size_t)c * 3 + j) * nlev + k];
-      const T ft = f * theta_e[ie];
-      dm += dv[j] * (double)f;
-      dt += dv[j] * (double)ft;
-    }
-    div_m[(size_t)c * nlev + k] = dm;
-    div_t[(size_t)c * nlev + k] = dt;
-  }
 }
 
 // -------------------------------------------------------------------------
@@ -1019,75 +911,49 @@ __global__ void sn_cell_fluxsum(GridT<double> g, VertT<double> v, const double* 
 }
 
 // -------------------------------------------------------------------------
-// Mixed mode: FP32 mirrors of the FP64 state at the start of a call
-// (the caller may have changed the state between calls).  One launch over
-// ne*nlev + nc*(nlev+1).
-// -------------------------------------------------------------------------
-__global__ void mx_refresh(int ne, int nc, int nlev, const double* __restrict__ exner_ref,
-                           const double* __restrict__ theta_ref, const double* __restrict__ rho_ref, StateView st,
-                           Mirrors m) {
-  const int nlevp = nlev + 1;
-  unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
-  const unsigned nedge = (unsigned)ne * nlev;
-  if (i < nedge) {
-    m.vn[i] = d2f(st.vn[i]);
-    return;
-  }
-  i -= nedge;
-  if (i >= (unsigned)nc * nlevp) return;
-  const int c = (int)(i / (unsigned)nlevp), k = (int)(i - (unsigned)c * nlevp);
-  m.w[i] = d2f(st.w[i]);
-  if (k < nlev) {
-    const size_t j = (size_t)c * nlev + k;
-    m.rho[j] = d2f(st.rho[j] - rho_ref[k]);
-    m.th[j] = d2f(st.theta_v[j] - theta_ref[k]);
-  }
-}
-
-// -------------------------------------------------------------------------
 // A10 diffusion
 // -------------------------------------------------------------------------
 // cells: div vn; vertices: curl vn and the vertex velocity (xyz)
-template <class T>
-__global__ void diff_div_curl_uv(GridT<T> g, VertT<T> v, const T* __restrict__ vn, T* __restrict__ div_vn,
-                                 T* __restrict__ zeta, T* __restrict__ uv3) {
+__global__ void diff_div_curl_uv(GridT<double> g, VertT<double> v, const double* __restrict__ vn,
+                                 double* __restrict__ div_vn, double* __restrict__ zeta, double* __restrict__ uv3) {
   const int nlev = v.nlev;
   unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
   const unsigned ncell = (unsigned)g.nc * nlev;
   if (i < ncell) {
     int c = (int)(i / (unsigned)nlev), k = (int)(i - (unsigned)c * nlev);
     const int* ce = g.c2e + 3 * (size_t)c;
-    const T* dv = g.div_c + 3 * (size_t)c;
-    div_vn[i] = dv[0] * vn[(size_t)ce[0] * nlev + k] + dv[1] * vn[(size_t)ce[1] * nlev + k] +
+    const double* dv = g.div_c + 3 * (size_t)c;
+    div_vn[(size_t)c * nlev + k] = dv[0] * vn[(size_t)ce[0] * nlev + k] + dv[1] * vn[(size_t)ce[1] * nlev + k] +
                 dv[2] * vn[(size_t)ce[2] * nlev + k];
     return;
   }
   i -= ncell;
-  const size_t nvl = (size_t)g.nv * nlev;
-  if (i >= nvl) return;
+  if (i >= (size_t)g.nv * nlev) return;
+  const size_t nvl = (size_t)g.nv * nlev;  // one plane of uv3
   int vx = (int)(i / (unsigned)nlev), k = (int)(i - (unsigned)vx * nlev);
   const int* ve = g.v2e + 6 * (size_t)vx;
-  const T* cw = g.curl_v + 6 * (size_t)vx;
-  const T* U = g.uv_w + 18 * (size_t)vx;
-  T z = 0, ux = 0, uy = 0, uz = 0;
+  const double* cw = g.curl_v + 6 * (size_t)vx;
+  const double* U = g.uv_w + 18 * (size_t)vx;
+  double z = 0, ux = 0, uy = 0, uz = 0;
 #pragma unroll
   for (int j = 0; j < 6; ++j) {
-    const T x = vn[(size_t)ve[j] * nlev + k];
+    const double x = vn[(size_t)ve[j] * nlev + k];
     z += cw[j] * x;
     ux += U[3 * j] * x;
     uy += U[3 * j + 1] * x;
     uz += U[3 * j + 2] * x;
   }
-  zeta[i] = z;
-  uv3[i] = ux;
-  uv3[nvl + i] = uy;
-  uv3[2 * nvl + i] = uz;
+  const size_t iv = (size_t)vx * nlev + k;
+  zeta[iv] = z;
+  uv3[iv] = ux;
+  uv3[nvl + iv] = uy;
+  uv3[2 * nvl + iv] = uz;
 }
 
 // edges: Smagorinsky coefficient and the vector Laplacian of vn
-template <class T>
-__global__ void diff_edge_smag(GridT<T> g, VertT<T> v, const T* __restrict__ div_vn, const T* __restrict__ zeta,
-                               const T* __restrict__ uv3, T* __restrict__ nu, T* __restrict__ lap) {
+__global__ void diff_edge_smag(GridT<double> g, VertT<double> v, const double* __restrict__ div_vn,
+                               const double* __restrict__ zeta, const double* __restrict__ uv3, double* __restrict__ nu,
+                               double* __restrict__ lap) {
   int e, k;
   const int nlev = v.nlev;
   if (!flat_index(g.ne, nlev, e, k)) return;
@@ -1095,12 +961,15 @@ __global__ void diff_edge_smag(GridT<T> g, VertT<T> v, const T* __restrict__ div
   const int* dm = g.e2c2v + 4 * (size_t)e;
   const size_t im = (size_t)dm[0] * nlev + k, ip = (size_t)dm[1] * nlev + k;
   const size_t i2 = (size_t)dm[2] * nlev + k, i3 = (size_t)dm[3] * nlev + k;
-  const T* nt = g.nt + 6 * (size_t)e;
-  const T dtx = uv3[ip] - uv3[im], dty = uv3[nvl + ip] - uv3[nvl + im], dtz = uv3[2 * nvl + ip] - uv3[2 * nvl + im];
-  const T dnx = uv3[i3] - uv3[i2], dny = uv3[nvl + i3] - uv3[nvl + i2], dnz = uv3[2 * nvl + i3] - uv3[2 * nvl + i2];
-  const T il = g.inv_l[e], idn = g.inv_dn[e];
-  const T tension = (dnx * nt[0] + dny * nt[1] + dnz * nt[2]) * idn - (dtx * nt[3] + dty * nt[4] + dtz * nt[5]) * il;
-  const T shear = (dtx * nt[0] + dty * nt[1] + dtz * nt[2]) * il + (dnx * nt[3] + dny * nt[4] + dnz * nt[5]) * idn;
+  const double* nt = g.nt + 6 * (size_t)e;
+  const double dtx = uv3[ip] - uv3[im], dty = uv3[nvl + ip] - uv3[nvl + im];
+  const double dtz = uv3[2 * nvl + ip] - uv3[2 * nvl + im];
+  const double dnx = uv3[i3] - uv3[i2], dny = uv3[nvl + i3] - uv3[nvl + i2];
+  const double dnz = uv3[2 * nvl + i3] - uv3[2 * nvl + i2];
+  const double il = g.inv_l[e], idn = g.inv_dn[e];
+  const double tension =
+      (dnx * nt[0] + dny * nt[1] + dnz * nt[2]) * idn - (dtx * nt[3] + dty * nt[4] + dtz * nt[5]) * il;
+  const double shear = (dtx * nt[0] + dty * nt[1] + dtz * nt[2]) * il + (dnx * nt[3] + dny * nt[4] + dnz * nt[5]) * idn;
   const size_t ie = (size_t)e * nlev + k;
   nu[ie] = g.smag_a[e] * sqrt(tension * tension + shear * shear);
   const int c0 = g.e2c[2 * e], c1 = g.e2c[2 * e + 1];
@@ -1110,11 +979,11 @@ __global__ void diff_edge_smag(GridT<T> g, VertT<T> v, const T* __restrict__ div
 
 // cells (half-level range): div of lap vn, cell Laplacian of w, theta increment;
 // vertices: curl of lap vn
-template <class T>
-__global__ void diff_second(GridT<T> g, VertT<T> v, ScalT<T> sc, const T* __restrict__ lap, const T* __restrict__ nu,
-                            const T* __restrict__ w, const T* __restrict__ theta, T* __restrict__ div_l,
-                            T* __restrict__ lap_w, T* __restrict__ dtheta, T* __restrict__ curl_l,
-                            const T* __restrict__ tenh_ex) {
+__global__ void diff_second(GridT<double> g, VertT<double> v, ScalT<double> sc, const double* __restrict__ lap,
+                            const double* __restrict__ nu, const double* __restrict__ w,
+                            const double* __restrict__ theta, double* __restrict__ div_l, double* __restrict__ lap_w,
+                            double* __restrict__ dtheta, double* __restrict__ curl_l,
+                            const double* __restrict__ tenh_ex) {
   const int nlev = v.nlev, nlevp = nlev + 1;
   unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
   const unsigned ncell = (unsigned)g.nc * nlevp;
@@ -1122,29 +991,29 @@ __global__ void diff_second(GridT<T> g, VertT<T> v, ScalT<T> sc, const T* __rest
     int c = (int)(i / (unsigned)nlevp), k = (int)(i - (unsigned)c * nlevp);
     const int* ce = g.c2e + 3 * (size_t)c;
     const int* cc = g.c2e2c + 3 * (size_t)c;
-    const T* L = g.lap_c + 3 * (size_t)c;
-    const T wc = w[(size_t)c * nlevp + k];
-    T lw = L[0] * (w[(size_t)cc[0] * nlevp + k] - wc);
+    const double* L = g.lap_c + 3 * (size_t)c;
+    const double wc = w[(size_t)c * nlevp + k];
+    double lw = L[0] * (w[(size_t)cc[0] * nlevp + k] - wc);
     lw += L[1] * (w[(size_t)cc[1] * nlevp + k] - wc);
     lw += L[2] * (w[(size_t)cc[2] * nlevp + k] - wc);
-    lap_w[i] = lw;
+    lap_w[(size_t)c * nlevp + k] = lw;
     if (k < nlev) {
-      const T* dv = g.div_c + 3 * (size_t)c;
+      const double* dv = g.div_c + 3 * (size_t)c;
       const size_t ic = (size_t)c * nlev + k;
       div_l[ic] = dv[0] * lap[(size_t)ce[0] * nlev + k] + dv[1] * lap[(size_t)ce[1] * nlev + k] +
                   dv[2] * lap[(size_t)ce[2] * nlev + k];
       if (sc.hdiff_temp) {
-        const T tc = theta[ic];
-        T n0 = nu[(size_t)ce[0] * nlev + k], n1 = nu[(size_t)ce[1] * nlev + k], n2 = nu[(size_t)ce[2] * nlev + k];
+        const double tc = theta[ic];
+        double n0 = nu[(size_t)ce[0] * nlev + k], n1 = nu[(size_t)ce[1] * nlev + k], n2 = nu[(size_t)ce[2] * nlev + k];
         if (k >= nlev - sc.tenh_levels) {
           // enhanced near-surface temperature diffusion: the edge coefficient
           // raised by fac A_e / dtime max(e_c, e_nbr)
-          const T ex = tenh_ex[ic];
+          const double ex = tenh_ex[ic];
           n0 += g.tenh_a[ce[0]] * max(ex, tenh_ex[(size_t)cc[0] * nlev + k]);
           n1 += g.tenh_a[ce[1]] * max(ex, tenh_ex[(size_t)cc[1] * nlev + k]);
           n2 += g.tenh_a[ce[2]] * max(ex, tenh_ex[(size_t)cc[2] * nlev + k]);
         }
-        T f = L[0] * n0 * (theta[(size_t)cc[0] * nlev + k] - tc);
+        double f = L[0] * n0 * (theta[(size_t)cc[0] * nlev + k] - tc);
         f += L[1] * n1 * (theta[(size_t)cc[1] * nlev + k] - tc);
         f += L[2] * n2 * (theta[(size_t)cc[2] * nlev + k] - tc);
         dtheta[ic] = sc.dtime * f;
@@ -1156,11 +1025,11 @@ __global__ void diff_second(GridT<T> g, VertT<T> v, ScalT<T> sc, const T* __rest
   if (i >= (unsigned)g.nv * nlev) return;
   int vx = (int)(i / (unsigned)nlev), k = (int)(i - (unsigned)vx * nlev);
   const int* ve = g.v2e + 6 * (size_t)vx;
-  const T* cw = g.curl_v + 6 * (size_t)vx;
-  T z = 0;
+  const double* cw = g.curl_v + 6 * (size_t)vx;
+  double z = 0;
 #pragma unroll
   for (int j = 0; j < 6; ++j) z += cw[j] * lap[(size_t)ve[j] * nlev + k];
-  curl_l[i] = z;
+  curl_l[(size_t)vx * nlev + k] = z;
 }
 
 // cells, the lowest tenh_levels levels: the excess factor of the enhanced
@@ -1171,81 +1040,57 @@ __global__ void diff_second(GridT<T> g, VertT<T> v, ScalT<T> sc, const T* __rest
 template <class T>
 __global__ void diff_tenh_excess(GridT<T> g, VertT<T> v, ScalT<T> sc, const T* __restrict__ theta,
                                  T* __restrict__ ex) {
-  const int nlev = v.nlev, nl = sc.tenh_levels;
+  const int nlev = v.nlev, ldf = v.ldf, nl = sc.tenh_levels;
   const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (unsigned)g.nc * (unsigned)nl) return;
   const int c = (int)(i / (unsigned)nl), k = nlev - nl + (int)(i - (unsigned)c * (unsigned)nl);
   const int* cc = g.c2e2c + 3 * (size_t)c;
-  const size_t ic = (size_t)c * nlev + k;
-  const T nbr = (theta[(size_t)cc[0] * nlev + k] + theta[(size_t)cc[1] * nlev + k] + theta[(size_t)cc[2] * nlev + k]) /
+  const size_t ic = (size_t)c * ldf + k;
+  const T nbr = (theta[(size_t)cc[0] * ldf + k] + theta[(size_t)cc[1] * ldf + k] + theta[(size_t)cc[2] * ldf + k]) /
                 T(3);
   const T x = (abs(theta[ic] - nbr) - sc.tenh_thresh) / sc.tenh_thresh;
   ex[ic] = x < T(0) ? T(0) : (x > T(1) ? T(1) : x);
 }
 
 // edges: vn update (FP64, in place)
-template <class T>
-__global__ void diff_edge_update(GridT<T> g, VertT<T> v, ScalT<T> sc, double* __restrict__ vn,
-                                 const T* __restrict__ nu, const T* __restrict__ lap, const T* __restrict__ div_l,
-                                 const T* __restrict__ curl_l, float* __restrict__ m_vn) {
+__global__ void diff_edge_update(GridT<double> g, VertT<double> v, ScalT<double> sc, double* __restrict__ vn,
+                                 const double* __restrict__ nu, const double* __restrict__ lap,
+                                 const double* __restrict__ div_l, const double* __restrict__ curl_l) {
   int e, k;
   const int nlev = v.nlev;
   if (!flat_index(g.ne, nlev, e, k)) return;
   const size_t ie = (size_t)e * nlev + k;
   const int c0 = g.e2c[2 * e], c1 = g.e2c[2 * e + 1];
   const int vm = g.e2v[2 * e], vp = g.e2v[2 * e + 1];
-  const T lap2 = (div_l[(size_t)c1 * nlev + k] - div_l[(size_t)c0 * nlev + k]) * g.inv_d[e] -
+  const double lap2 = (div_l[(size_t)c1 * nlev + k] - div_l[(size_t)c0 * nlev + k]) * g.inv_d[e] -
                  (curl_l[(size_t)vp * nlev + k] - curl_l[(size_t)vm * nlev + k]) * g.inv_l[e];
-  const T inc = sc.dtime * nu[ie] * lap[ie] - g.k4_a[e] * lap2;
-  if constexpr (kMixed<T>) {
-    const double vnn = vn[ie] + f2d(inc);
-    vn[ie] = vnn;
-    m_vn[ie] = d2f(vnn);
-  } else {
-    vn[ie] = vn[ie] + (double)inc;
-  }
+  const double inc = sc.dtime * nu[ie] * lap[ie] - g.k4_a[e] * lap2;
+  vn[ie] = vn[ie] + (double)inc;
 }
 
 // cells (half-level range): w fourth-order diffusion, theta/exner update (FP64, in place)
-template <class T>
-__global__ void diff_cell_update(GridT<T> g, VertT<T> v, ScalT<T> sc, const double* __restrict__ theta_ref,
-                                 const double* __restrict__ exner_ref, double rd_o_cvd, StateView st,
-                                 const T* __restrict__ lap_w, const T* __restrict__ dtheta, Mirrors m) {
+__global__ void diff_cell_update(GridT<double> g, VertT<double> v, ScalT<double> sc, double rd_o_cvd, StateView st,
+                                 const double* __restrict__ lap_w, const double* __restrict__ dtheta) {
   int c, k;
   const int nlev = v.nlev, nlevp = nlev + 1;
   if (!flat_index(g.nc, nlevp, c, k)) return;
   if (k > 0 && k < nlev) {
     const int* cc = g.c2e2c + 3 * (size_t)c;
-    const T* L = g.lap_c + 3 * (size_t)c;
-    const T lc = lap_w[(size_t)c * nlevp + k];
-    T l2 = L[0] * (lap_w[(size_t)cc[0] * nlevp + k] - lc);
+    const double* L = g.lap_c + 3 * (size_t)c;
+    const double lc = lap_w[(size_t)c * nlevp + k];
+    double l2 = L[0] * (lap_w[(size_t)cc[0] * nlevp + k] - lc);
     l2 += L[1] * (lap_w[(size_t)cc[1] * nlevp + k] - lc);
     l2 += L[2] * (lap_w[(size_t)cc[2] * nlevp + k] - lc);
     const size_t iw = (size_t)c * nlevp + k;
-    if constexpr (kMixed<T>) {
-      const double wn = st.w[iw] - f2d(g.k4w_c[c] * l2);
-      st.w[iw] = wn;
-      m.w[iw] = d2f(wn);
-    } else {
-      st.w[iw] = st.w[iw] - (double)(g.k4w_c[c] * l2);
-    }
+    st.w[iw] = st.w[iw] - (double)(g.k4w_c[c] * l2);
   }
   if (k < nlev && sc.hdiff_temp) {
     const size_t ic = (size_t)c * nlev + k;
     const double th = st.theta_v[ic];
-    if constexpr (kMixed<T>) {
-      // exner (1 + rd/cvd dtheta/theta): the FP32 increment of a value near 1
-      const float dth = dtheta[ic];
-      const double thn = th + f2d(dth);
-      st.theta_v[ic] = thn;
-      st.exner[ic] = st.exner[ic] + f2d(d2f(st.exner[ic]) * ((float)rd_o_cvd * dth / d2f(th)));
-      m.th[ic] = d2f(thn - theta_ref[k]);
-    } else {
-      const double thn = th + (double)dtheta[ic];
-      const double exn = st.exner[ic] * (1.0 + rd_o_cvd * (thn - th) / th);
-      st.theta_v[ic] = thn;
-      st.exner[ic] = exn;
-    }
+    const double thn = th + (double)dtheta[ic];
+    const double exn = st.exner[ic] * (1.0 + rd_o_cvd * (thn - th) / th);
+    st.theta_v[ic] = thn;
+    st.exner[ic] = exn;
   }
 }
 
@@ -1254,6 +1099,15 @@ __global__ void diff_cell_update(GridT<T> g, VertT<T> v, ScalT<T> sc, const doub
 // -------------------------------------------------------------------------
 // launch sequences
 // -------------------------------------------------------------------------
+namespace {
+// whether rows of nlev FP64 values of these arrays can be read two at a time
+bool aligned_pairs(int nlev, std::initializer_list<const double*> arrays) {
+  size_t bits = 0;
+  for (const double* p : arrays) bits |= reinterpret_cast<size_t>(p);
+  return nlev % 2 == 0 && bits % 16 == 0;
+}
+}  // namespace
+
 template <class T>
 void launch_velocity_tendencies(const Ctx<T>& x, const T* vn, const T* w, T* ddt_vn, T* ddt_w, const T* divd,
                                 T* divd2, cudaStream_t s, const int* threads, T* wcc, const int* shapes) {
@@ -1272,27 +1126,42 @@ void launch_velocity_tendencies(const Ctx<T>& x, const T* vn, const T* w, T* ddt
                        ddt_vn, ddt_w, divd, divd2);
       return;
     }
-  }
-  ICON_LAUNCH(kname<T>("va_edge_pre", "va_edge_pre_f32"), blocks_by_shape(SH(0), g.ne, nlev, TH(0)), TH(0), s,
-              va_edge_pre<T>, g, v, vn, wk.vt, wk.ekin_e, wk.vn_ie, terr ? tr.wgt_e : nullptr, SH(0));
-  if (terr)
-    ICON_LAUNCH(kname<T>("va_concorr", "va_concorr_f32"), blocks_for((long long)g.nc * nlevp, TH(14)), TH(14), s,
-                va_concorr<T>, g, v, tr, wk.vn_ie, wk.vt, wcc);
-  const long long n2 = (long long)g.nc * nlev + (long long)g.nv * nlevp;
-  ICON_LAUNCH(kname<T>("va_cell_vert", "va_cell_vert_f32"), blocks_for(n2, TH(1)), TH(1), s, va_cell_vert<T>, g,
-              v, vn, w, wk.ekin_e, wk.ekin_c, divd, divd2, wk.zeta, wk.w_v, wk.wq, terr ? (const T*)wcc : nullptr);
-  if (terr) {
-    ICON_LAUNCH(kname<T>("va_edge_tend_terrain", "va_edge_tend_terrain_f32"),
-                blocks_for((long long)g.ne * nlevp, TH(2)), TH(2), s, (va_edge_tend<T, true>), g, v, wk.vn_ie, w, wk.vt,
-                wk.ekin_c, wk.zeta, wk.w_v, ddt_vn, wk.gw_e, tr, (const T*)wk.wq);
-    ICON_LAUNCH(kname<T>("va_cell_w_terrain", "va_cell_w_terrain_f32"), blocks_by_shape(SH(3), g.nc, nlevp, TH(3)),
-                TH(3), s, (va_cell_w<T, true>), g, v, w, wk.gw_e, ddt_w, tr, wcc, SH(3));
+    // four levels per thread
+    const long long nqf = quads_full(nlev), nqh = quads_half(nlev);
+    T* const q_wcc = terr ? wcc : nullptr;
+    ICON_LAUNCH("va_edge_pre_f32", blocks_for(g.ne * nqf, TH(0)), TH(0), s, va_edge_pre_q, g, v, vn, wk.vt, wk.ekin_e,
+                wk.vn_ie, terr ? tr.wgt_e : nullptr);
+    if (terr)
+      ICON_LAUNCH("va_concorr_f32", blocks_for(g.nc * nqh, TH(14)), TH(14), s, va_concorr_q, g, v, tr, wk.vn_ie,
+                  wk.vt, wcc);
+    ICON_LAUNCH("va_cell_vert_f32", blocks_for(g.nc * nqf + g.nv * nqh, TH(1)), TH(1), s, va_cell_vert_q, g, v, vn, w,
+                wk.ekin_e, wk.ekin_c, divd, divd2, wk.zeta, wk.w_v, wk.wq, q_wcc);
+    const char* const nm_tend = terr ? "va_edge_tend_terrain_f32" : "va_edge_tend_f32";
+    const char* const nm_w = terr ? "va_cell_w_terrain_f32" : "va_cell_w_f32";
+    ICON_LAUNCH(nm_tend, blocks_for(g.ne * nqh, TH(2)), TH(2), s, (terr ? va_edge_tend_q<true> : va_edge_tend_q<false>),
+                g, v, wk.vn_ie, w, wk.vt, wk.ekin_c, wk.zeta, wk.w_v, ddt_vn, wk.gw_e, tr, wk.wq);
+    ICON_LAUNCH(nm_w, blocks_for(g.nc * nqh, TH(3)), TH(3), s, (terr ? va_cell_w_q<true> : va_cell_w_q<false>), g, v,
+                w, wk.gw_e, ddt_w, tr, q_wcc);
   } else {
-    ICON_LAUNCH(kname<T>("va_edge_tend", "va_edge_tend_f32"), blocks_for((long long)g.ne * nlevp, TH(2)), TH(2),
-                s, (va_edge_tend<T, false>), g, v, wk.vn_ie, w, wk.vt, wk.ekin_c, wk.zeta, wk.w_v, ddt_vn, wk.gw_e, tr,
-                (const T*)wk.wq);
-    ICON_LAUNCH(kname<T>("va_cell_w", "va_cell_w_f32"), blocks_by_shape(SH(3), g.nc, nlevp, TH(3)), TH(3), s,
-                (va_cell_w<T, false>), g, v, w, wk.gw_e, ddt_w, tr, wcc, SH(3));
+    ICON_LAUNCH("va_edge_pre", blocks_by_shape(SH(0), g.ne, nlev, TH(0)), TH(0), s, va_edge_pre, g, v, vn, wk.vt,
+                wk.ekin_e, wk.vn_ie, terr ? tr.wgt_e : nullptr, SH(0));
+    if (terr)
+      ICON_LAUNCH("va_concorr", blocks_for((long long)g.nc * nlevp, TH(14)), TH(14), s, va_concorr, g, v, tr,
+                  wk.vn_ie, wk.vt, wcc);
+    const long long n2 = (long long)g.nc * nlev + (long long)g.nv * nlevp;
+    ICON_LAUNCH("va_cell_vert", blocks_for(n2, TH(1)), TH(1), s, va_cell_vert, g, v, vn, w, wk.ekin_e, wk.ekin_c, divd,
+                divd2, wk.zeta, wk.w_v, wk.wq, terr ? (const T*)wcc : nullptr);
+    if (terr) {
+      ICON_LAUNCH("va_edge_tend_terrain", blocks_for((long long)g.ne * nlevp, TH(2)), TH(2), s, va_edge_tend<true>, g,
+                  v, wk.vn_ie, w, wk.vt, wk.ekin_c, wk.zeta, wk.w_v, ddt_vn, wk.gw_e, tr, (const T*)wk.wq);
+      ICON_LAUNCH("va_cell_w_terrain", blocks_by_shape(SH(3), g.nc, nlevp, TH(3)), TH(3), s, va_cell_w<true>, g, v, w,
+                  wk.gw_e, ddt_w, tr, wcc, SH(3));
+    } else {
+      ICON_LAUNCH("va_edge_tend", blocks_for((long long)g.ne * nlevp, TH(2)), TH(2), s, va_edge_tend<false>, g, v,
+                  wk.vn_ie, w, wk.vt, wk.ekin_c, wk.zeta, wk.w_v, ddt_vn, wk.gw_e, tr, (const T*)wk.wq);
+      ICON_LAUNCH("va_cell_w", blocks_by_shape(SH(3), g.nc, nlevp, TH(3)), TH(3), s, va_cell_w<false>, g, v, w,
+                  wk.gw_e, ddt_w, tr, wcc, SH(3));
+    }
   }
 }
 
@@ -1307,8 +1176,9 @@ void launch_fluxdiv(const Engine& en, const Ctx<T>& x, const T* vn, const char* 
   const WorkT<T>& wk = x.w;
   const int nlev = v.nlev;
   if constexpr (kMixed<T>) {
-    ICON_LAUNCH(name, blocks_by_point<T>(g.nc, nlev, TH(7)), TH(7), s, (sn_cell_fluxdiv<T, kTerr>), g, v, x.s, vn,
-                wk.divd, wk.rho_e, wk.theta_e, en.g64.div_c, en.wk.div_m, en.wk.div_t, x.tr.fx_ratio);
+    ICON_LAUNCH(name, blocks_for((long long)g.nc * quads_full(nlev), TH(7)), TH(7), s, sn_cell_fluxdiv_q<kTerr>, g, v,
+                vn, wk.divd, wk.rho_e, wk.theta_e, reinterpret_cast<df*>(en.wk.div_m),
+                reinterpret_cast<df*>(en.wk.div_t), x.tr.fx_ratio);
   } else {
     ICON_LAUNCH("sn_edge_flux", blocks_for((long long)g.ne * nlev, TH(15)), TH(15), s, sn_edge_flux, g, v, vn,
                 wk.divd, wk.rho_e, wk.theta_e, wk.flx_m, wk.flx_t);
@@ -1344,8 +1214,10 @@ void substep_impl(const Engine& en, const Ctx<T>& x, const StateView& st, cudaSt
   const TerrT<T>& tr = x.tr;
   const Mirrors& m = en.m;
   const int nlev = v.nlev;
-  const long long nce = (long long)g.nc * nlev, nee = (long long)g.ne * nlev;
+  const long long nce = (long long)g.nc * nlev, nee = (long long)g.ne * nlev, nqf = quads_full(nlev);
   const double* ex_ref_c = en.v.exner_ref_c;
+  // the caller's FP64 rows in aligned pairs of levels (the quad kernels)
+  const bool pairs = aligned_pairs(nlev, {st.exner, st.exner_pr});
   // stencil views of the state: the FP64 state itself, or the FP32 mirrors
   const T *s_vn, *s_w, *s_rho, *s_th, *s_wp;
   if constexpr (kMixed<T>) {
@@ -1365,16 +1237,32 @@ void substep_impl(const Engine& en, const Ctx<T>& x, const StateView& st, cudaSt
   launch_velocity_tendencies<T>(x, s_vn, s_w, wk.ddt_vn0, wk.ddt_w0, nullptr, nullptr, s, threads,
                                 kTerr ? tr.wcc0 : nullptr, shapes);
   if (en.io_wait) stream_wait_io(s, en.io_wait);  // rho, theta_v, exner, exner_pr from here on
-  ICON_LAUNCH(nm_grad, blocks_for(nce, TH(4)), TH(4), s, (sn_cell_grad<T, kTerr>), g, v, s_rho, s_th, wk.grad4,
-              st.exner, st.exner_pr, en.sc.exfac, en.wk.pex, ex_ref_c);
-  ICON_LAUNCH(nm_pred, blocks_for(nee, TH(5)), TH(5), s, (sn_edge_pred<T, kTerr>), g, v, x.s, s_vn, wk.vt,
-              wk.ddt_vn0, s_rho, s_th, en.wk.pex, en.g64.cpd_inv_d, wk.grad4, wk.rho_e, wk.theta_e, wk.hpg, wk.vn_p, tr);
+  if constexpr (kMixed<T>) {
+    ICON_LAUNCH(nm_grad, blocks_for(g.nc * nqf, TH(4)), TH(4), s, sn_cell_grad_q<kTerr>, g, v, s_rho, s_th, wk.grad4,
+                st.exner, st.exner_pr, en.sc.exfac, reinterpret_cast<df*>(en.wk.pex), ex_ref_c, pairs);
+    ICON_LAUNCH(nm_pred, blocks_for(g.ne * nqf, TH(5)), TH(5), s, sn_edge_pred_q<kTerr>, g, v, x.s, s_vn, wk.vt,
+                wk.ddt_vn0, s_rho, s_th, reinterpret_cast<const df*>(en.wk.pex), wk.grad4, wk.rho_e, wk.theta_e,
+                wk.hpg, wk.vn_p, tr);
+  } else {
+    ICON_LAUNCH(nm_grad, blocks_for(nce, TH(4)), TH(4), s, sn_cell_grad<kTerr>, g, v, s_rho, s_th, wk.grad4, st.exner,
+                st.exner_pr, en.sc.exfac, en.wk.pex, ex_ref_c);
+    ICON_LAUNCH(nm_pred, blocks_for(nee, TH(5)), TH(5), s, sn_edge_pred<kTerr>, g, v, x.s, s_vn, wk.vt, wk.ddt_vn0,
+                s_rho, s_th, en.wk.pex, en.g64.cpd_inv_d, wk.grad4, wk.rho_e, wk.theta_e, wk.hpg, wk.vn_p, tr);
+  }
   if (kTerr && en.v.n_steep > 0)
     ICON_LAUNCH(kname<T>("sn_edge_hpg_steep", "sn_edge_hpg_steep_f32"), blocks_for(en.v.n_steep, 128), 128, s,
                 sn_edge_hpg_steep<T>, g, v, x.s, en.v.n_steep, en.v.steep_idx, en.v.steep_w, en.wk.pex,
                 en.v.exner_ref_c, en.g64.cpd_inv_d, wk.theta_e, s_vn, wk.ddt_vn0, wk.hpg, wk.vn_p);
-  ICON_LAUNCH(nm_div, blocks_by_shape(SH(6), g.nc, nlev, TH(6)), TH(6), s, (sn_cell_div<T, kTerr>), g, v, wk.vn_p,
-              wk.divd, st.exner, st.exner_pr, ex_ref_c, SH(6));
+  // divergence of a velocity field; the predictor's call also updates the exner history
+  auto cell_div = [&](const T* vn, double* exner_pr) {
+    if constexpr (kMixed<T>)
+      ICON_LAUNCH(nm_div, blocks_for(g.nc * nqf, TH(6)), TH(6), s, sn_cell_div_q<kTerr>, g, v, vn, wk.divd, st.exner,
+                  exner_pr, ex_ref_c, pairs);
+    else
+      ICON_LAUNCH(nm_div, blocks_by_shape(SH(6), g.nc, nlev, TH(6)), TH(6), s, sn_cell_div<kTerr>, g, v, vn, wk.divd,
+                  st.exner, exner_pr, ex_ref_c, SH(6));
+  };
+  cell_div(wk.vn_p, st.exner_pr);
   launch_fluxdiv<T, kTerr>(en, x, wk.vn_p, nm_flx, s);
   if constexpr (kTerr)
     launch_column_terrain<T>(en, 0, st, wk.ddt_w0, wk.ddt_w1, tr.wcc0, s);
@@ -1386,8 +1274,7 @@ void substep_impl(const Engine& en, const Ctx<T>& x, const StateView& st, cudaSt
   ICON_LAUNCH(kname<T>("sn_edge_corr", "sn_edge_corr_f32"), blocks_by_shape(SH(8), g.ne, nlev, TH(8)), TH(8), s,
               sn_edge_corr<T>, g, v, x.s, st.vn, wk.ddt_vn0, wk.ddt_vn1, wk.hpg, wk.divd2, m.vn, SH(8));
   const T* vn_new = kMixed<T> ? (const T*)m.vn : (const T*)st.vn;
-  ICON_LAUNCH(nm_div, blocks_by_shape(SH(6), g.nc, nlev, TH(6)), TH(6), s, (sn_cell_div<T, kTerr>), g, v, vn_new,
-              wk.divd, nullptr, nullptr, ex_ref_c, SH(6));
+  cell_div(vn_new, nullptr);
   launch_fluxdiv<T, kTerr>(en, x, vn_new, nm_flx, s);
   if constexpr (kTerr)
     launch_column_terrain<T>(en, 1, st, wk.ddt_w0, wk.ddt_w1, tr.wcc1, s);
@@ -1417,23 +1304,40 @@ void launch_diffusion(const Engine& en, const Ctx<T>& x, const StateView& st, cu
   } else {
     s_vn = st.vn, s_w = st.w, s_th = st.theta_v;
   }
-  const long long n1 = (long long)g.nc * nlev + (long long)g.nv * nlev;
-  ICON_LAUNCH(kname<T>("diff_div_curl_uv", "diff_div_curl_uv_f32"), blocks_for(n1, TH(9)), TH(9), s,
-              diff_div_curl_uv<T>, g, v, s_vn, wk.div_vn, wk.zeta, wk.uv3);
-  ICON_LAUNCH(kname<T>("diff_edge_smag", "diff_edge_smag_f32"), blocks_for((long long)g.ne * nlev, TH(10)),
-              TH(10), s, diff_edge_smag<T>, g, v, wk.div_vn, wk.zeta, wk.uv3, wk.nu, wk.lap_vn);
+  const long long nqf = quads_full(nlev), nqh = quads_half(nlev);
+  const long long n1 = (long long)(g.nc + g.nv) * nlev;
+  const long long n3 = (long long)g.nc * nlevp + (long long)g.nv * nlev;
+  if constexpr (kMixed<T>) {  // four levels per thread
+    ICON_LAUNCH("diff_div_curl_uv_f32", blocks_for((g.nc + g.nv) * nqf, TH(9)), TH(9), s, diff_div_curl_uv_q, g, v,
+                s_vn, wk.div_vn, wk.zeta, wk.uv3);
+    ICON_LAUNCH("diff_edge_smag_f32", blocks_for(g.ne * nqf, TH(10)), TH(10), s, diff_edge_smag_q, g, v, wk.div_vn,
+                wk.zeta, wk.uv3, wk.nu, wk.lap_vn);
+  } else {
+    ICON_LAUNCH("diff_div_curl_uv", blocks_for(n1, TH(9)), TH(9), s, diff_div_curl_uv, g, v, s_vn, wk.div_vn, wk.zeta,
+                wk.uv3);
+    ICON_LAUNCH("diff_edge_smag", blocks_for((long long)g.ne * nlev, TH(10)), TH(10), s, diff_edge_smag, g, v,
+                wk.div_vn, wk.zeta, wk.uv3, wk.nu, wk.lap_vn);
+  }
   if (x.s.tenh_levels > 0 && x.s.hdiff_temp)
     ICON_LAUNCH(kname<T>("diff_tenh_excess", "diff_tenh_excess_f32"),
                 blocks_for((long long)g.nc * x.s.tenh_levels, kThreads), kThreads, s, diff_tenh_excess<T>, g, v, x.s,
                 s_th, wk.tenh_ex);
-  const long long n3 = (long long)g.nc * nlevp + (long long)g.nv * nlev;
-  ICON_LAUNCH(kname<T>("diff_second", "diff_second_f32"), blocks_for(n3, TH(11)), TH(11), s, diff_second<T>, g, v,
-              x.s, wk.lap_vn, wk.nu, s_w, s_th, wk.div_l, wk.lap_w, wk.dtheta, wk.curl_l, wk.tenh_ex);
-  ICON_LAUNCH(kname<T>("diff_edge_update", "diff_edge_update_f32"), blocks_for((long long)g.ne * nlev, TH(12)),
-              TH(12), s, diff_edge_update<T>, g, v, x.s, st.vn, wk.nu, wk.lap_vn, wk.div_l, wk.curl_l, m.vn);
-  ICON_LAUNCH(kname<T>("diff_cell_update", "diff_cell_update_f32"), blocks_for((long long)g.nc * nlevp, TH(13)),
-              TH(13), s, diff_cell_update<T>, g, v, x.s, en.v.theta_ref, en.v.exner_ref, en.sc.rd_o_cvd, st,
-              wk.lap_w, wk.dtheta, m);
+  if constexpr (kMixed<T>) {
+    ICON_LAUNCH("diff_second_f32", blocks_for(g.nc * nqh + g.nv * nqf, TH(11)), TH(11), s, diff_second_q, g, v, x.s,
+                wk.lap_vn, wk.nu, s_w, s_th, wk.div_l, wk.lap_w, wk.dtheta, wk.curl_l, wk.tenh_ex);
+    ICON_LAUNCH("diff_edge_update_f32", blocks_for(g.ne * nqf, TH(12)), TH(12), s, diff_edge_update_q, g, v, x.s,
+                st.vn, wk.nu, wk.lap_vn, wk.div_l, wk.curl_l, m.vn, aligned_pairs(nlev, {st.vn}));
+    ICON_LAUNCH("diff_cell_update_f32", blocks_for(g.nc * nqh, TH(13)), TH(13), s, diff_cell_update_q, g, v, x.s,
+                en.v.theta_ref, en.sc.rd_o_cvd, st, wk.lap_w, wk.dtheta, m,
+                aligned_pairs(nlev, {st.theta_v, st.exner}));
+  } else {
+    ICON_LAUNCH("diff_second", blocks_for(n3, TH(11)), TH(11), s, diff_second, g, v, x.s, wk.lap_vn, wk.nu, s_w, s_th,
+                wk.div_l, wk.lap_w, wk.dtheta, wk.curl_l, wk.tenh_ex);
+    ICON_LAUNCH("diff_edge_update", blocks_for((long long)g.ne * nlev, TH(12)), TH(12), s, diff_edge_update, g, v,
+                x.s, st.vn, wk.nu, wk.lap_vn, wk.div_l, wk.curl_l);
+    ICON_LAUNCH("diff_cell_update", blocks_for((long long)g.nc * nlevp, TH(13)), TH(13), s, diff_cell_update, g, v,
+                x.s, en.sc.rd_o_cvd, st, wk.lap_w, wk.dtheta);
+  }
 }
 
 namespace {
@@ -1460,9 +1364,9 @@ const char* const kStencilNames[kNumStencils] = {
 
 void launch_refresh_mirrors(const Engine& en, const StateView& st, cudaStream_t s) {
   const int nlev = en.v.nlev;
-  const long long n = (long long)en.g64.ne * nlev + (long long)en.g64.nc * (nlev + 1);
-  ICON_LAUNCH("mx_refresh", blocks_for(n, kThreads), kThreads, s, mx_refresh, en.g64.ne, en.g64.nc, nlev,
-              en.v.exner_ref, en.v.theta_ref, en.rho_ref64, st, en.m);
+  const long long n = (long long)en.g64.ne * quads_full(nlev) + (long long)en.g64.nc * quads_half(nlev);
+  ICON_LAUNCH("mx_refresh", blocks_for(n, kThreads), kThreads, s, mx_refresh, en.g64.ne, en.g64.nc, en.c32.v,
+              en.v.theta_ref, en.rho_ref64, st, en.m, aligned_pairs(nlev, {st.vn, st.rho, st.theta_v}));
 }
 
 template void launch_velocity_tendencies<double>(const Ctx<double>&, const double*, const double*, double*, double*,
