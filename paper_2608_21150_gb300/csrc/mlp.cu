@@ -451,87 +451,167 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc(const __grid_constant__
   }
 }
 
-// out[c][r] = in[r][c] for r < rows, c < cols (bf16); pads of out left untouched
-__global__ void transpose_bf16(int rows, int cols, const __nv_bfloat16* __restrict__ in, int ldi,
-                               __nv_bfloat16* __restrict__ out, int ldo) {
-  __shared__ __nv_bfloat16 tile[32][33];
-  const int c = blockIdx.x * 32 + threadIdx.x, r0 = blockIdx.y * 32;
-  for (int j = threadIdx.y; j < 32; j += blockDim.y) {
-    const int r = r0 + j;
-    if (r < rows && c < cols) tile[j][threadIdx.x] = in[(size_t)r * ldi + c];
+// Before a layer's weight-gradient GEMM, one launch: the bias gradient
+// db[c] = sum_r dz[r][c] (the first blocks, 32 columns each) and the transposes
+// dz^T and h^T (the other blocks, 64 x 64 tiles), which run beside it.
+//
+// The bias sum keeps one sequential FP32 sum per column, so it is bound by that
+// chain of adds (4 cycles a row: 8 us at 4096 rows): the block's threads stage
+// 128-row tiles in shared memory with cp.async, two ahead, and one warp adds.
+// At 4096 rows of 512 columns 11 us with both transposes; with one thread per
+// column reading global memory row by row it took 125 us, waiting for each
+// load, and the transposes 18 us in launches of their own.
+constexpr int kPrepThreads = 256, kSumRows = 128, kSumStages = 3, kTr = 64;
+struct PrepArgs {
+  int rows;                    // a multiple of 64
+  const float* dz32;           // [rows][ldz], ldz a multiple of 64
+  const __nv_bfloat16* dz16;   // [rows][ldz]
+  int ldz, cols;
+  float* db;                   // [cols]
+  __nv_bfloat16* dzT;          // [cols][ldt]
+  const __nv_bfloat16* h;      // [rows][ldh]
+  int ldh, hcols;
+  __nv_bfloat16* hT;           // [hcols][ldt]
+  int ldt;                     // a multiple of 8
+};
+__device__ __forceinline__ void cp16(void* smem, const void* g) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(g)
+               : "memory");
+}
+__global__ void __launch_bounds__(kPrepThreads) layer_prep(PrepArgs a) {
+  __shared__ __align__(16) unsigned char raw[kSumStages * kSumRows * 32 * sizeof(float)];
+  const int tid = threadIdx.x, nsum = (a.cols + 31) / 32;
+  int bid = blockIdx.x;
+  if (bid < nsum) {
+    auto tile = reinterpret_cast<float(*)[kSumRows][32]>(raw);
+    const int c0 = 32 * bid, nt = (a.rows + kSumRows - 1) / kSumRows;
+    auto stage = [&](int t) {
+      if (t < nt) {
+        const int n = min(kSumRows, a.rows - t * kSumRows) * 8;  // 16-byte pieces
+        for (int i = tid; i < n; i += kPrepThreads)
+          cp16(&tile[t % kSumStages][i >> 3][4 * (i & 7)],
+               a.dz32 + (size_t)(t * kSumRows + (i >> 3)) * a.ldz + c0 + 4 * (i & 7));
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    stage(0);
+    stage(1);
+    float sum = 0.f;
+    for (int t = 0; t < nt; ++t) {
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+      __syncthreads();  // tile t has landed; its predecessor's buffer is read
+      stage(t + 2);
+      if (tid < 32) {
+        const int n = min(kSumRows, a.rows - t * kSumRows);  // a multiple of 64
+        for (int r0 = 0; r0 < n; r0 += 64) {
+#pragma unroll
+          for (int r = 0; r < 64; ++r) sum += tile[t % kSumStages][r0 + r][tid];
+        }
+      }
+    }
+    if (tid < 32 && c0 + tid < a.cols) a.db[c0 + tid] = sum;
+    return;
+  }
+  bid -= nsum;
+  const int rt = a.rows / kTr, nz = rt * ((a.cols + kTr - 1) / kTr);
+  const bool is_h = bid >= nz;
+  if (is_h) bid -= nz;
+  const __nv_bfloat16* in = is_h ? a.h : a.dz16;
+  __nv_bfloat16* out = is_h ? a.hT : a.dzT;
+  const int ld = is_h ? a.ldh : a.ldz, cols = is_h ? a.hcols : a.cols;
+  const int r0 = (bid % rt) * kTr, c0 = (bid / rt) * kTr;
+  // rows of 33 words: both the row-wise writes and the column-wise reads touch every bank once
+  auto tr = reinterpret_cast<uint32_t(*)[kTr / 2 + 1]>(raw);
+#pragma unroll
+  for (int i = tid; i < kTr * 8; i += kPrepThreads) {
+    const uint4 x = *reinterpret_cast<const uint4*>(in + (size_t)(r0 + (i >> 3)) * ld + c0 + 8 * (i & 7));
+    uint32_t* q = &tr[i >> 3][4 * (i & 7)];
+    q[0] = x.x, q[1] = x.y, q[2] = x.z, q[3] = x.w;
   }
   __syncthreads();
-  const int rr = r0 + threadIdx.x;
-  for (int j = threadIdx.y; j < 32; j += blockDim.y) {
-    const int cc = blockIdx.x * 32 + j;
-    if (rr < rows && cc < cols) out[(size_t)cc * ldo + rr] = tile[threadIdx.x][j];
+#pragma unroll
+  for (int i = tid; i < kTr * 8; i += kPrepThreads) {
+    // lanes: 4 groups of eight rows by 8 columns
+    const int g = (i & 3) + 4 * ((i >> 5) & 1), c = ((i >> 2) & 7) + 8 * (i >> 6);
+    uint32_t v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      v[j] = __byte_perm(tr[8 * g + 2 * j][c >> 1], tr[8 * g + 2 * j + 1][c >> 1], c & 1 ? 0x7632 : 0x5410);
+    if (c0 + c < cols)
+      *reinterpret_cast<uint4*>(out + (size_t)(c0 + c) * a.ldt + r0 + 8 * g) = make_uint4(v[0], v[1], v[2], v[3]);
   }
 }
+
+// The elementwise passes below: one warp per row, lanes over the columns (with
+// a flat index the 64-bit division by the row length took longer than the
+// values: 14 -> 4 us at 4096 x 512).
+constexpr int kRowWarps = 8;
 
 // dZ = dH * gelu'(Z) (bf16 out for the next GEMMs, fp32 kept for the bias gradient)
 __global__ void gelu_backward(int rows, int cols, const float* __restrict__ dh, int ldd,
                               const float* __restrict__ z, int ldz, float* __restrict__ dz32,
                               __nv_bfloat16* __restrict__ dz16, int ldo) {
-  const size_t n = (size_t)rows * cols;
-  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int r = (int)(i / cols), c = (int)(i - (size_t)r * cols);
-  const float v = dh[(size_t)r * ldd + c] * gelu_grad(z[(size_t)r * ldz + c]);
-  dz32[(size_t)r * ldo + c] = v;
-  dz16[(size_t)r * ldo + c] = __float2bfloat16(v);
+  const int r = blockIdx.x * kRowWarps + (threadIdx.x >> 5);
+  if (r >= rows) return;
+#pragma unroll 4
+  for (int c = threadIdx.x & 31; c < cols; c += 32) {
+    const float v = dh[(size_t)r * ldd + c] * gelu_grad(z[(size_t)r * ldz + c]);
+    dz32[(size_t)r * ldo + c] = v;
+    dz16[(size_t)r * ldo + c] = __float2bfloat16(v);
+  }
 }
 
 // fp32 -> bf16 copy with padding (pads written as zero)
 __global__ void to_bf16(int rows, int cols, const float* __restrict__ in, int ldi, __nv_bfloat16* __restrict__ out,
                         int ldo) {
-  const size_t n = (size_t)rows * ldo;
-  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int r = (int)(i / ldo), c = (int)(i - (size_t)r * ldo);
-  out[i] = __float2bfloat16(c < cols ? in[(size_t)r * ldi + c] : 0.f);
+  const int r = blockIdx.x * kRowWarps + (threadIdx.x >> 5);
+  if (r >= rows) return;
+#pragma unroll 4
+  for (int c = threadIdx.x & 31; c < ldo; c += 32)
+    out[(size_t)r * ldo + c] = __float2bfloat16(c < cols ? in[(size_t)r * ldi + c] : 0.f);
 }
 
-// db[c] = sum_r dz[r][c], fixed order per column (one thread per column)
-__global__ void bias_grad(int rows, int cols, const float* __restrict__ dz, int ldd, float* __restrict__ db) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= cols) return;
-  float s = 0.f;
-  for (int r = 0; r < rows; ++r) s += dz[(size_t)r * ldd + c];
-  db[c] = s;
+// Adam on the fp32 master weights and biases of the three layers, one launch;
+// refreshes the bf16 copies W^T [n_out][ldt] and W [n_in][ldw].  A block takes
+// a 32 x 32 tile of one layer's weights, so that both copies are written in
+// runs (W through shared memory: 2-byte stores ldw apart took a sector each),
+// the last blocks of a layer its biases.  At 512 x 512: three layers and their
+// biases 8 us instead of 43 in six launches.
+__device__ __forceinline__ float adam_value(const AdamScal& q, float w, float gi, float& m, float& v) {
+  const float mi = q.b1 * m + (1.f - q.b1) * gi;
+  const float vi = q.b2 * v + (1.f - q.b2) * gi * gi;
+  m = mi;
+  v = vi;
+  return w - q.lr * (mi / q.c1) / (sqrtf(vi / q.c2) + q.eps);
 }
-
-// Adam on fp32 master weights; refreshes the bf16 copy W^T [n][k] and W [k][n]
-__global__ void adam_update(int n_out, int n_in, float* __restrict__ w, const float* __restrict__ g,
-                            float* __restrict__ m, float* __restrict__ v, float lr, float b1, float b2, float eps,
-                            float c1, float c2, __nv_bfloat16* __restrict__ wt16, int ldt,
-                            __nv_bfloat16* __restrict__ w16, int ldw) {
-  const size_t n = (size_t)n_out * n_in;
-  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float gi = g[i];
-  const float mi = b1 * m[i] + (1.f - b1) * gi;
-  const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-  w[i] = wi;
-  if (wt16) {
-    const int o = (int)(i / n_in), k = (int)(i - (size_t)o * n_in);
-    wt16[(size_t)o * ldt + k] = __float2bfloat16(wi);
-    w16[(size_t)k * ldw + o] = __float2bfloat16(wi);
+__global__ void __launch_bounds__(256) adam_update(AdamLayers ly, AdamScal q) {
+  __shared__ __nv_bfloat16 tile[32][34];
+  int l = 0;
+  while (l < 2 && (int)blockIdx.x >= ly.l[l].block_end) ++l;
+  const AdamLayer& a = ly.l[l];
+  const int bid = (int)blockIdx.x - (l ? ly.l[l - 1].block_end : 0);
+  const int tk = (a.n_in + 31) / 32, nt = tk * ((a.n_out + 31) / 32);
+  if (bid >= nt) {
+    const int i = (bid - nt) * 256 + threadIdx.x;
+    if (i < a.n_out) a.b[i] = adam_value(q, a.b[i], a.gb[i], a.mb[i], a.vb[i]);
+    return;
   }
-}
-
-__global__ void adam_update_bias(int n, float* __restrict__ b, const float* __restrict__ g, float* __restrict__ m,
-                                 float* __restrict__ v, float lr, float b1, float b2, float eps, float c1, float c2) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float gi = g[i];
-  const float mi = b1 * m[i] + (1.f - b1) * gi;
-  const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  b[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  const int k0 = (bid % tk) * 32, o0 = (bid / tk) * 32, x = threadIdx.x & 31, y = threadIdx.x >> 5;
+#pragma unroll
+  for (int j = y; j < 32; j += 8) {
+    const int o = o0 + j, k = k0 + x;
+    if (o >= a.n_out || k >= a.n_in) continue;
+    const size_t i = (size_t)o * a.n_in + k;
+    const float wi = adam_value(q, a.w[i], a.gw[i], a.mw[i], a.vw[i]);
+    a.w[i] = wi;
+    const __nv_bfloat16 h = __float2bfloat16(wi);
+    a.wt16[(size_t)o * a.ldt + k] = h;
+    tile[j][x] = h;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int j = y; j < 32; j += 8)
+    if (k0 + j < a.n_in && o0 + x < a.n_out) a.w16[(size_t)(k0 + j) * a.ldw + o0 + x] = tile[x][j];
 }
 
 inline unsigned cdiv(size_t a, size_t b) { return (unsigned)((a + b - 1) / b); }
@@ -605,61 +685,68 @@ const int* mlp_tc_error_flag() {
   return static_cast<const int*>(p);
 }
 
-void mlp_transpose(int rows, int cols, const __nv_bfloat16* in, int ldi, __nv_bfloat16* out, int ldo,
-                   cudaStream_t s) {
-  dim3 grid(cdiv(cols, 32), cdiv(rows, 32));
-  ICON_LAUNCH("mlp_transpose", grid, dim3(32, 8), s, transpose_bf16, rows, cols, in, ldi, out, ldo);
+void mlp_layer_prep(int rows, int cols, const float* dz32, const __nv_bfloat16* dz16, int ldz, float* db,
+                    __nv_bfloat16* dzT, int hcols, const __nv_bfloat16* h, int ldh, __nv_bfloat16* hT, int ldt,
+                    cudaStream_t s) {
+  const PrepArgs a{rows, dz32, dz16, ldz, cols, db, dzT, h, ldh, hcols, hT, ldt};
+  const unsigned grid = cdiv(cols, 32) + (unsigned)(rows / kTr) * (cdiv(cols, kTr) + cdiv(hcols, kTr));
+  ICON_LAUNCH("mlp_layer_prep", grid, kPrepThreads, s, layer_prep, a);
 }
 
 void mlp_gelu_backward(int rows, int cols, const float* dh, int ldd, const float* z, int ldz, float* dz32,
                        __nv_bfloat16* dz16, int ldo, cudaStream_t s) {
-  ICON_LAUNCH("mlp_gelu_backward", cdiv((size_t)rows * cols, 256), 256, s, gelu_backward, rows, cols, dh, ldd, z,
-              ldz, dz32, dz16, ldo);
+  ICON_LAUNCH("mlp_gelu_backward", cdiv(rows, kRowWarps), 32 * kRowWarps, s, gelu_backward, rows, cols, dh, ldd, z, ldz,
+              dz32, dz16, ldo);
 }
 
 void mlp_to_bf16(int rows, int cols, const float* in, int ldi, __nv_bfloat16* out, int ldo, cudaStream_t s) {
-  ICON_LAUNCH("mlp_to_bf16", cdiv((size_t)rows * ldo, 256), 256, s, to_bf16, rows, cols, in, ldi, out, ldo);
+  ICON_LAUNCH("mlp_to_bf16", cdiv(rows, kRowWarps), 32 * kRowWarps, s, to_bf16, rows, cols, in, ldi, out, ldo);
 }
 
-void mlp_bias_grad(int rows, int cols, const float* dz, int ldd, float* db, cudaStream_t s) {
-  ICON_LAUNCH("mlp_bias_grad", cdiv(cols, 128), 128, s, bias_grad, rows, cols, dz, ldd, db);
-}
-
-void mlp_adam(int n_out, int n_in, float* w, const float* g, float* m, float* v, float lr, float b1, float b2,
-              float eps, float c1, float c2, __nv_bfloat16* wt16, int ldt, __nv_bfloat16* w16, int ldw,
-              cudaStream_t s) {
-  ICON_LAUNCH("mlp_adam", cdiv((size_t)n_out * n_in, 256), 256, s, adam_update, n_out, n_in, w, g, m, v, lr, b1, b2,
-              eps, c1, c2, wt16, ldt, w16, ldw);
-}
-
-void mlp_adam_bias(int n, float* b, const float* g, float* m, float* v, float lr, float b1, float b2, float eps,
-                   float c1, float c2, cudaStream_t s) {
-  ICON_LAUNCH("mlp_adam_bias", cdiv(n, 256), 256, s, adam_update_bias, n, b, g, m, v, lr, b1, b2, eps, c1, c2);
+void mlp_adam(AdamLayers& ly, const AdamScal& q, cudaStream_t s) {
+  int n = 0;
+  for (AdamLayer& a : ly.l) {
+    n += (int)(cdiv(a.n_in, 32) * cdiv(a.n_out, 32) + cdiv(a.n_out, 256));
+    a.block_end = n;
+  }
+  ICON_LAUNCH("mlp_adam", (unsigned)n, 256, s, adam_update, ly, q);
 }
 
 }  // namespace icon
 
 namespace icon {
 namespace {
+// One warp per row; dy, its bf16 copy (pads zero) and the row's FP64 loss, whose
+// two FP64 operations a value bound it (4096 rows of 361: 62 us with one thread
+// per row -> 7).
 __global__ void mse_kernel(int B, int n_out, const float* __restrict__ y, int ldy, const float* __restrict__ t,
-                           int ldt, float* __restrict__ dy, int lddy, double* __restrict__ rowloss) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+                           int ldt, float* __restrict__ dy, __nv_bfloat16* __restrict__ dy16, int lddy,
+                           double* __restrict__ rowloss) {
+  const int r = blockIdx.x * kRowWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (r >= B) return;
   const float scale = 2.0f / ((float)B * (float)n_out);
   double s = 0.0;
-  for (int c = 0; c < n_out; ++c) {
-    const float d = y[(size_t)r * ldy + c] - t[(size_t)r * ldt + c];
-    s += (double)d * d;
-    dy[(size_t)r * lddy + c] = scale * d;
+#pragma unroll 4
+  for (int c = lane; c < lddy; c += 32) {
+    float v = 0.f;
+    if (c < n_out) {
+      const float d = y[(size_t)r * ldy + c] - t[(size_t)r * ldt + c];
+      s += (double)d * d;
+      v = scale * d;
+      dy[(size_t)r * lddy + c] = v;
+    }
+    dy16[(size_t)r * lddy + c] = __float2bfloat16(v);
   }
-  rowloss[r] = s;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(~0u, s, o);
+  if (lane == 0) rowloss[r] = s;
 }
 }  // namespace
 
-void mlp_mse(int B, int n_out, const float* y, int ldy, const float* t, int ldt, float* dy, int lddy, double* rowloss,
-             cudaStream_t s) {
-  ICON_LAUNCH("mlp_mse", (unsigned)((B + 127) / 128), 128, s, mse_kernel, B, n_out, y, ldy, t, ldt, dy, lddy,
-              rowloss);
+void mlp_mse(int B, int n_out, const float* y, int ldy, const float* t, int ldt, float* dy, __nv_bfloat16* dy16,
+             int lddy, double* rowloss, cudaStream_t s) {
+  ICON_LAUNCH("mlp_mse", (unsigned)((B + kRowWarps - 1) / kRowWarps), 32 * kRowWarps, s, mse_kernel, B, n_out, y, ldy,
+              t, ldt, dy, dy16, lddy, rowloss);
 }
 
 }  // namespace icon

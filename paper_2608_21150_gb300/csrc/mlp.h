@@ -16,21 +16,33 @@ namespace icon {
 int mlp_gemm(int M, int N, int K, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb,
               const float* bias, bool gelu_act, float* out_f32, __nv_bfloat16* out_bf16, float* zpre, int ldc,
               cudaStream_t s);
-void mlp_transpose(int rows, int cols, const __nv_bfloat16* in, int ldi, __nv_bfloat16* out, int ldo,
-                   cudaStream_t s);
+// db[c] = sum_r dz32[r][c] (one sequential FP32 sum per column), dzT = dz16^T and
+// hT = h^T (columns below cols / hcols).  rows and the leading dimensions of the
+// inputs are multiples of 64, ldt (>= rows) of 8; bases on 16 bytes.
+void mlp_layer_prep(int rows, int cols, const float* dz32, const __nv_bfloat16* dz16, int ldz, float* db,
+                    __nv_bfloat16* dzT, int hcols, const __nv_bfloat16* h, int ldh, __nv_bfloat16* hT, int ldt,
+                    cudaStream_t s);
 void mlp_gelu_backward(int rows, int cols, const float* dh, int ldd, const float* z, int ldz, float* dz32,
                        __nv_bfloat16* dz16, int ldo, cudaStream_t s);
 void mlp_to_bf16(int rows, int cols, const float* in, int ldi, __nv_bfloat16* out, int ldo, cudaStream_t s);
-void mlp_bias_grad(int rows, int cols, const float* dz, int ldd, float* db, cudaStream_t s);
-void mlp_adam(int n_out, int n_in, float* w, const float* g, float* m, float* v, float lr, float b1, float b2,
-              float eps, float c1, float c2, __nv_bfloat16* wt16, int ldt, __nv_bfloat16* w16, int ldw,
-              cudaStream_t s);
-void mlp_adam_bias(int n, float* b, const float* g, float* m, float* v, float lr, float b1, float b2, float eps,
-                   float c1, float c2, cudaStream_t s);
+struct AdamLayer {
+  int n_out, n_in, ldt, ldw, block_end;
+  float *w, *b;
+  const float *gw, *gb;
+  float *mw, *vw, *mb, *vb;
+  __nv_bfloat16 *wt16, *w16;
+};
+struct AdamLayers {
+  AdamLayer l[3];
+};
+struct AdamScal {
+  float lr, b1, b2, eps, c1, c2;
+};
+void mlp_adam(AdamLayers& ly, const AdamScal& q, cudaStream_t s);  // fills block_end
 // loss = sum (y - t)^2 / (B n_out) (per-row partial sums into rowloss[B]);
-// dy = 2 (y - t) / (B n_out)
-void mlp_mse(int B, int n_out, const float* y, int ldy, const float* t, int ldt, float* dy, int lddy, double* rowloss,
-             cudaStream_t s);
+// dy = 2 (y - t) / (B n_out), and its bf16 copy with zero pads
+void mlp_mse(int B, int n_out, const float* y, int ldy, const float* t, int ldt, float* dy, __nv_bfloat16* dy16,
+             int lddy, double* rowloss, cudaStream_t s);
 
 // Device address of the tensor-core GEMM's error word (nonzero once a GEMM gave
 // up a bounded wait; sticky).

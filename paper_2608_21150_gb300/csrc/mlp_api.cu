@@ -100,20 +100,17 @@ int forward(icon_mlp* m, const float* x, int B, cudaStream_t s, bool keep_z = tr
   return forward_from(m, m->x16, m->lds[0], B, s, keep_z);
 }
 
-// gradients of all parameters for dL/dy in m->dy (fp32 [B][lds[3]]), after
-// forward(); B a multiple of 64 (the K extent of the weight-gradient GEMMs)
+// gradients of all parameters for dL/dy in m->dy (fp32 [B][lds[3]]) and m->dz16
+// (its bf16 copy), after forward(); B a multiple of 64 (the K extent of the
+// weight-gradient GEMMs)
 int backward(icon_mlp* m, int B, cudaStream_t s) {
-  // layer 3 (no activation): dz = dy
-  const int n3 = layer_out(m, 2);
-  mlp_to_bf16(B, n3, m->dy, m->lds[3], m->dz16, m->lds[3], s);
-  mlp_bias_grad(B, n3, m->dy, m->lds[3], m->gb[2], s);
+  const float* dz32 = m->dy;  // layer 3 (no activation): dz = dy
   int ldz = m->lds[3];
   for (int l = 2; l >= 0; --l) {
     const int nin = layer_in(m, l), nout = layer_out(m, l);
     const __nv_bfloat16* h = l == 0 ? m->x16 : m->h16[l - 1];
     // dW^T [nout][nin] = dZ^T H over the batch
-    mlp_transpose(B, nout, m->dz16, ldz, m->dzT, m->ld_b, s);
-    mlp_transpose(B, nin, h, m->lds[l], m->hT, m->ld_b, s);
+    mlp_layer_prep(B, nout, dz32, m->dz16, ldz, m->gb[l], m->dzT, nin, h, m->lds[l], m->hT, m->ld_b, s);
     int rc = mlp_gemm(nout, nin, B, m->dzT, m->ld_b, m->hT, m->ld_b, nullptr, false, m->gw[l], nullptr, nullptr, nin,
                       s);
     if (rc != ICON_OK) return rc;
@@ -124,7 +121,7 @@ int backward(icon_mlp* m, int B, cudaStream_t s) {
     if (rc != ICON_OK) return rc;
     // dZ of the previous layer through its GELU
     mlp_gelu_backward(B, nin, m->dh, m->lds[l], m->z[l - 1], m->lds[l], m->dz32, m->dz16, m->lds[l], s);
-    mlp_bias_grad(B, nin, m->dz32, m->lds[l], m->gb[l - 1], s);
+    dz32 = m->dz32;
     ldz = m->lds[l];
   }
   return ICON_OK;
@@ -132,13 +129,12 @@ int backward(icon_mlp* m, int B, cudaStream_t s) {
 
 void adam(icon_mlp* m, float lr, float b1, float b2, float eps, cudaStream_t s) {
   m->adam_t += 1;
-  const float c1 = 1.f - std::pow(b1, (float)m->adam_t), c2 = 1.f - std::pow(b2, (float)m->adam_t);
-  for (int l = 0; l < 3; ++l) {
-    const int nin = layer_in(m, l), nout = layer_out(m, l);
-    mlp_adam(nout, nin, m->w[l], m->gw[l], m->mw[l], m->vw[l], lr, b1, b2, eps, c1, c2, m->wt16[l], m->lds[l],
-             m->w16[l], m->lds[l + 1], s);
-    mlp_adam_bias(nout, m->b[l], m->gb[l], m->mb[l], m->vb[l], lr, b1, b2, eps, c1, c2, s);
-  }
+  const AdamScal q{lr, b1, b2, eps, 1.f - std::pow(b1, (float)m->adam_t), 1.f - std::pow(b2, (float)m->adam_t)};
+  AdamLayers ly;
+  for (int l = 0; l < 3; ++l)
+    ly.l[l] = {layer_out(m, l), layer_in(m, l), m->lds[l], m->lds[l + 1], 0,          m->w[l],  m->b[l],   m->gw[l],
+               m->gb[l],        m->mw[l],       m->vw[l],  m->mb[l],      m->vb[l], m->wt16[l], m->w16[l]};
+  mlp_adam(ly, q, s);
 }
 
 __global__ void refresh_bf16(int n_out, int n_in, const float* __restrict__ w, __nv_bfloat16* __restrict__ wt16,
@@ -415,6 +411,7 @@ int icon_mlp_backward(icon_mlp_t* m, const float* dy, int32_t batch, void* strea
   if (cudaMemcpy2DAsync(m->dy, m->lds[3] * 4, dy, m->dims[3] * 4, m->dims[3] * 4, batch, cudaMemcpyDeviceToDevice,
                         s) != cudaSuccess)
     return fail_m(ICON_ERR_CUDA, "icon_mlp_backward: copy failed");
+  mlp_to_bf16(batch, m->dims[3], m->dy, m->lds[3], m->dz16, m->lds[3], s);
   rc = backward(m, batch, s);
   if (rc != ICON_OK) return rc;
   cudaError_t e = cudaStreamSynchronize(s);
@@ -437,7 +434,8 @@ int icon_mlp_train_step(icon_mlp_t* m, const float* x, const float* target, int3
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   rc = forward(m, x, batch, s);
   if (rc != ICON_OK) return rc;
-  mlp_mse(batch, m->dims[3], m->y, m->lds[3], target, m->dims[3], m->dy, m->lds[3], m->rowloss, s);
+  mlp_mse(batch, m->dims[3], m->y, m->lds[3], target, m->dims[3], m->dy, m->dz16, m->lds[3],
+          m->rowloss, s);
   rc = backward(m, batch, s);
   if (rc != ICON_OK) return rc;
   adam(m, lr, 0.9f, 0.999f, 1e-8f, s);
