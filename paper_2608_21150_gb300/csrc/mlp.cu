@@ -57,15 +57,22 @@ __device__ __forceinline__ float gelu_fwd(float x) {
 // 2..9 drain the other accumulator meanwhile (TMEM -> registers -> bias, GELU,
 // stores): warp w may access TMEM lanes 32 (w % 4) .. +31 (= tile rows), and
 // the two warps of a lane quarter split the columns.
-constexpr int TBM = 128, TBN = 128, TBK = 64, kStages = 5;
+//
+// A product with few tiles and a long K (a weight gradient: 512 x 512 over 4096
+// rows, 16 tiles of 64 K blocks) is bound by what one SM can load, 32 KB a K
+// block: tiles of 128 x 32 load 20 KB and put four times the SMs to work.  The
+// order of the sums over K is the same.
+constexpr int TBM = 128, TBK = 64;
+constexpr int kWideN = 128, kWideStages = 5, kSlimN = 32, kSlimStages = 8;
 constexpr int kEpiWarps = 8;
 constexpr int kTcThreads = 64 + 32 * kEpiWarps;
-constexpr int kTileBytesA = TBM * TBK * 2, kTileBytesB = TBN * TBK * 2;
+constexpr int kTileBytesA = TBM * TBK * 2;
 // per epilogue warp, a staging block of its 32 rows x 64 columns of BF16 output
 constexpr int kStageBytes = 32 * 64 * 2;
-constexpr int kTcSmem = kStages * (kTileBytesA + kTileBytesB) + kEpiWarps * kStageBytes +
-                        1024 /* alignment slack */ + 256 /* barriers */;
-constexpr uint32_t kTmemCols = 2 * TBN;
+constexpr int tc_smem(int n, int stages) {
+  return stages * (kTileBytesA + n * TBK * 2) + kEpiWarps * kStageBytes + 1024 /* alignment slack */ +
+         256 /* barriers */;
+}
 // every wait gives up after this long (ns) and flags an error instead of hanging
 constexpr unsigned long long kWaitLimitNs = 1000000000ull;
 
@@ -236,9 +243,13 @@ __device__ __forceinline__ void epilogue16(float (&v)[16], int row, int col0, in
   }
 }
 
+template <int TBN, int kStages>
 __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc(const __grid_constant__ CUtensorMap tma_a,
                                                          const __grid_constant__ CUtensorMap tma_b, int M, int N,
                                                          int K, Epi ep) {
+  constexpr int kTileBytesB = TBN * TBK * 2;
+  constexpr uint32_t kTmemCols = 2 * TBN;
+  constexpr bool kStagedOut = TBN == 128;  // the staged stores below move 64-column halves
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sA = base;
@@ -340,7 +351,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc(const __grid_constant__
       const int row = m0 + 32 * quarter + lane;
       const uint32_t trow = tmem + (uint32_t)(b * TBN) + ((uint32_t)(32 * quarter) << 16);
       const int cw = n0 + half * (TBN / 2);  // first column of this warp's half
-      if (ep.mode == 1 && !ep.zpre && cw + TBN / 2 <= N && (ep.ldc & 1) == 0 &&
+      if (kStagedOut && ep.mode == 1 && !ep.zpre && cw + TBN / 2 <= N && (ep.ldc & 1) == 0 &&
           (reinterpret_cast<uintptr_t>(ep.out_bf16) & 3) == 0) {
         // GELU to BF16 staged in this warp's block (row = lane, 16-byte chunks
         // XOR-swizzled by the row so that 8 lanes writing one chunk hit all
@@ -381,7 +392,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc(const __grid_constant__
           if (grow < M) *reinterpret_cast<uint32_t*>(ep.out_bf16 + (size_t)grow * ep.ldc + cw + 2 * lane) = val;
         }
         __syncwarp();
-      } else if (ep.mode == 0 && cw + TBN / 2 <= N) {
+      } else if (kStagedOut && ep.mode == 0 && cw + TBN / 2 <= N) {
         // FP32 (+ bias) staged the same way, 32 columns (128 bytes a row) at a time
         uint8_t* st = sOut + (warp - 2) * kStageBytes;
 #pragma unroll 1
@@ -661,7 +672,10 @@ int mlp_gemm(int M, int N, int K, const __nv_bfloat16* A, int lda, const __nv_bf
   {
     std::lock_guard<std::mutex> lk(g_attr_mutex);
     if (!g_attr_set[dev]) {
-      if (cudaFuncSetAttribute(gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem) != cudaSuccess)
+      if (cudaFuncSetAttribute(gemm_tc<kWideN, kWideStages>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               tc_smem(kWideN, kWideStages)) != cudaSuccess ||
+          cudaFuncSetAttribute(gemm_tc<kSlimN, kSlimStages>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               tc_smem(kSlimN, kSlimStages)) != cudaSuccess)
         return report_error(ICON_ERR_CUDA, "mlp_gemm: shared memory attribute");
       if (cudaDeviceGetAttribute(&g_sm_count[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
           g_sm_count[dev] < 1)
@@ -669,13 +683,22 @@ int mlp_gemm(int M, int N, int K, const __nv_bfloat16* A, int lda, const __nv_bf
       g_attr_set[dev] = true;
     }
   }
+  // the slim tiles while four of them still find an idle SM each
+  const long long wide = (long long)cdiv(N, kWideN) * cdiv(M, TBM);
+  const bool slim = 4 * wide <= g_sm_count[dev];
+  const int tn = slim ? kSlimN : kWideN;
   CUtensorMap ta, tb;
-  if (!operand_map(&ta, A, M, K, lda, TBM) || !operand_map(&tb, B, N, K, ldb, TBN))
+  if (!operand_map(&ta, A, M, K, lda, TBM) || !operand_map(&tb, B, N, K, ldb, tn))
     return report_error(ICON_ERR_CUDA, "mlp_gemm: tensor map encoding failed");
   Epi ep{gelu_act ? 1 : 0, bias, out_f32, out_bf16, zpre, ldc};
-  const long long tiles = (long long)cdiv(N, TBN) * cdiv(M, TBM);
+  const long long tiles = (long long)cdiv(N, tn) * cdiv(M, TBM);
   const unsigned grid = (unsigned)std::min<long long>(tiles, g_sm_count[dev]);  // one persistent CTA per SM
-  ICON_LAUNCH_SMEM("mlp_gemm_tc", grid, kTcThreads, kTcSmem, s, gemm_tc, ta, tb, M, N, K, ep);
+  if (slim)
+    ICON_LAUNCH_SMEM("mlp_gemm_tc", grid, kTcThreads, tc_smem(kSlimN, kSlimStages), s,
+                     (gemm_tc<kSlimN, kSlimStages>), ta, tb, M, N, K, ep);
+  else
+    ICON_LAUNCH_SMEM("mlp_gemm_tc", grid, kTcThreads, tc_smem(kWideN, kWideStages), s,
+                     (gemm_tc<kWideN, kWideStages>), ta, tb, M, N, K, ep);
   return ICON_OK;
 }
 
