@@ -253,6 +253,33 @@ void release_streams(icon_dycore* d) {
 int create_dycore(const icon_grid_t* grid, int nlev, const double* z_ifc, const double* z_cols,
                   const icon_dycore_params_t* p, icon_dycore_t** out, const char* fn);
 
+// Basis of a cell's gradient sum_j G_j (psi_j - psi_c), G [3][2]: nb = (a, b, m)
+// with the least parallel pair (a, b) and b4 = (alpha, beta, 1 + alpha, 1 + beta),
+// G_m = alpha G_a + beta G_b.  Where no pair spans the plane, G_m along the
+// longest vector.
+void grad_basis(const double* G, int* nb, double* b4) {
+  auto det = [&](int i, int j) { return G[2 * i] * G[2 * j + 1] - G[2 * i + 1] * G[2 * j]; };
+  int m = 2;
+  for (int j = 0; j < 2; ++j)
+    if (std::fabs(det((j + 1) % 3, (j + 2) % 3)) > std::fabs(det((m + 1) % 3, (m + 2) % 3))) m = j;
+  int a = (m + 1) % 3, b = (m + 2) % 3;
+  double al = 0.0, be = 0.0;
+  const double d = det(a, b);
+  if (d != 0.0) {
+    al = det(m, b) / d;
+    be = det(a, m) / d;
+  } else {
+    auto dot = [&](int i, int j) { return G[2 * i] * G[2 * j] + G[2 * i + 1] * G[2 * j + 1]; };
+    for (int j = 0; j < 3; ++j)
+      if (dot(j, j) > dot(a, a)) a = j;
+    b = (a + 1) % 3;
+    m = (a + 2) % 3;
+    if (dot(a, a) > 0.0) al = dot(m, a) / dot(a, a);
+  }
+  nb[0] = a, nb[1] = b, nb[2] = m;
+  b4[0] = al, b4[1] = be, b4[2] = 1.0 + al, b4[3] = 1.0 + be;
+}
+
 // Autotuner: time every kernel of one step on a temporary uniform state with
 // each candidate launch shape (CUDA events around every launch) and keep the
 // fastest shape per kernel.
@@ -264,9 +291,10 @@ bool grid_complete(const GridT<T>& g) {
   const void* p[] = {g.c2e, g.c2e2c, g.e2c, g.e2v, g.e2c2v, g.e2c2e, g.v2e, g.v2c, g.div_c, g.lap_c, g.e2c_w,
                      g.grad_c, g.k4w_c, g.inv_d, g.inv_l, g.f_e, g.vt_w, g.upw, g.nt, g.inv_dn, g.smag_a, g.k4_a,
                      g.fdiv_e, g.ddamp_e, g.curl_v, g.c2v_w, g.uv_w, g.cell_area, g.uv_c, g.div_c_hl,
-                     g.upw_s, g.cpd_inv_d, g.hinv_d, g.d_o_l, g.grad_s, g.lap_s, g.e2c_wd};
+                     g.upw_s, g.cpd_inv_d, g.hinv_d, g.d_o_l, g.lap_s, g.e2c_wd};
   for (const void* q : p)
     if (!q) return false;
+  if (std::is_same<T, double>::value && (!g.grad_nb || !g.grad_b || !g.smag_c)) return false;
   return true;
 }
 
@@ -526,7 +554,7 @@ int create_dycore(const icon_grid_t* grid, int nlev, const double* z_ifc, const 
   for (int c = 0; c < nc; ++c) k4w[c] = p->hdiff_w_k4 * h.cell_area[c] * h.cell_area[c];
   // dycore-level factors of the predictor's edge kernel: upwind offsets with
   // the half-substep scaling folded in, and cpd / d_e
-  std::vector<double> upw_s(h.upw), cid(ne), tenh(ne);
+  std::vector<double> upw_s(h.upw), cid(ne), tenh(ne), tenh64(ne);
   for (int e = 0; e < ne; ++e) tenh[e] = p->hdiff_tenh_fac * h.edge_area[e] / p->dtime;
   const bool tenh_on = p->hdiff_temp && p->hdiff_tenh_fac > 0.0 && p->hdiff_tenh_levels > 0;
   for (int e = 0; e < ne; ++e) {
@@ -536,7 +564,7 @@ int create_dycore(const icon_grid_t* grid, int nlev, const double* z_ifc, const 
   }
   // factors that fold constants of the stencils into stored products (fewer
   // FP64 operations per point-level)
-  std::vector<double> hinv_d(ne), d_o_l(ne), grad_s(2 * (size_t)nc, 0.0), lap_s(nc, 0.0), e2c_wd(3 * (size_t)nc);
+  std::vector<double> hinv_d(ne), d_o_l(ne), lap_s(nc, 0.0), e2c_wd(3 * (size_t)nc);
   for (int e = 0; e < ne; ++e) {
     hinv_d[e] = 0.5 * h.inv_d[e];
     d_o_l[e] = h.inv_l[e] / h.inv_d[e];
@@ -544,20 +572,44 @@ int create_dycore(const icon_grid_t* grid, int nlev, const double* z_ifc, const 
   for (int c = 0; c < nc; ++c)
     for (int j = 0; j < 3; ++j) {
       const size_t cj = 3 * (size_t)c + j;
-      grad_s[2 * (size_t)c] += h.grad_c[2 * cj];
-      grad_s[2 * (size_t)c + 1] += h.grad_c[2 * cj + 1];
       lap_s[c] += h.lap_c[cj];
       e2c_wd[cj] = h.e2c_w[cj] * h.inv_d[h.c2e[cj]];
     }
+  // FP64: the gradient in two of its three vectors (GridT), the upwind offsets
+  // in that basis, and the factors of the Smagorinsky coefficient
+  std::vector<int> grad_nb(3 * (size_t)nc);
+  std::vector<double> grad_b(4 * (size_t)nc), upw_b(upw_s), smag_c(12 * (size_t)ne);
+  for (int c = 0; c < nc; ++c) grad_basis(&h.grad_c[6 * (size_t)c], &grad_nb[3 * (size_t)c], &grad_b[4 * (size_t)c]);
+  for (int e = 0; e < ne; ++e) {
+    for (int side = 0; side < 2; ++side) {
+      const int c = h.e2c[2 * (size_t)e + side];
+      const double* Ga = &h.grad_c[6 * (size_t)c + 2 * grad_nb[3 * (size_t)c]];
+      const double* Gb = &h.grad_c[6 * (size_t)c + 2 * grad_nb[3 * (size_t)c + 1]];
+      for (int j = 0; j < 6; j += 2) {
+        const double* u = &upw_s[12 * (size_t)e + 6 * side + j];
+        upw_b[12 * (size_t)e + 6 * side + j] = u[0] * Ga[0] + u[1] * Ga[1];
+        upw_b[12 * (size_t)e + 6 * side + j + 1] = u[0] * Gb[0] + u[1] * Gb[1];
+      }
+    }
+    const double a = std::fabs(smag[e]) * p->dtime;
+    const double f[4] = {a * h.inv_dn[e], a * h.inv_l[e], a * h.inv_l[e], a * h.inv_dn[e]};
+    for (int j = 0; j < 12; ++j) smag_c[12 * (size_t)e + j] = f[j / 3] * h.nt[6 * (size_t)e + j % 6];
+    tenh64[e] = p->hdiff_tenh_fac * h.edge_area[e];
+  }
+  // cells by their place in the connectivity, as the kernel reads them
+  for (int c = 0; c < nc; ++c)
+    for (int j = 0; j < 3; ++j) grad_nb[3 * (size_t)c + j] = h.c2e2c[3 * (size_t)c + grad_nb[3 * (size_t)c + j]];
   en.g64 = grid->dev;
   en.g64.hinv_d = A.upload(hinv_d);
   en.g64.d_o_l = A.upload(d_o_l);
-  en.g64.grad_s = A.upload(grad_s);
+  en.g64.grad_nb = A.upload(grad_nb);
+  en.g64.grad_b = A.upload(grad_b);
+  en.g64.smag_c = A.upload(smag_c);
   en.g64.lap_s = A.upload(lap_s);
   en.g64.e2c_wd = A.upload(e2c_wd);
-  en.g64.upw_s = A.upload(upw_s);
+  en.g64.upw_s = A.upload(upw_b);
   en.g64.cpd_inv_d = A.upload(cid);
-  en.g64.tenh_a = tenh_on ? A.upload(tenh) : nullptr;
+  en.g64.tenh_a = tenh_on ? A.upload(tenh64) : nullptr;
   en.g64.f_e = A.upload(fe);
   en.g64.smag_a = A.upload(smag);
   en.g64.k4_a = A.upload(k4);
@@ -602,7 +654,6 @@ int create_dycore(const icon_grid_t* grid, int nlev, const double* z_ifc, const 
     g.inv_l = up(h.inv_l);
     g.hinv_d = up(hinv_d);
     g.d_o_l = up(d_o_l);
-    g.grad_s = up(grad_s);
     g.lap_s = up(lap_s);
     g.e2c_wd = up(e2c_wd);
     g.f_e = up(fe);
@@ -1410,6 +1461,25 @@ int icon_dycore_debug_field(icon_dycore_t* d, const char* name, void* dst, int64
   if (bytes < (int64_t)n) return fail(ICON_ERR_ARG, "icon_dycore_debug_field: destination too small");
   CUDA_TRY(cudaMemcpy2DAsync(dst, width, src, pitch, width, rows, cudaMemcpyDeviceToDevice, d->stream));
   CUDA_TRY(cudaStreamSynchronize(d->stream));
+  if (!mixed && std::strcmp(name, "grad4") == 0) {
+    // from the cells' own basis to the x and y of their frames
+    const size_t plane = nc * nlev;
+    std::vector<double> f(4 * plane);
+    CUDA_TRY(cudaMemcpy(f.data(), dst, n, cudaMemcpyDeviceToHost));
+    for (size_t c = 0; c < nc; ++c) {
+      int nb[3];
+      double b4[4];
+      const double* G = &h.grad_c[6 * c];
+      grad_basis(G, nb, b4);
+      for (size_t i = c * nlev; i < (c + 1) * nlev; ++i)
+        for (double* p = &f[i]; p <= &f[2 * plane + i]; p += 2 * plane) {
+          const double ga = p[0], gb = p[plane];
+          p[0] = G[2 * nb[0]] * ga + G[2 * nb[1]] * gb;
+          p[plane] = G[2 * nb[0] + 1] * ga + G[2 * nb[1] + 1] * gb;
+        }
+    }
+    CUDA_TRY(cudaMemcpy(dst, f.data(), n, cudaMemcpyHostToDevice));
+  }
   return ICON_OK;
 }
 

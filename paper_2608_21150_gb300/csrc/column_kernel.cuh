@@ -37,11 +37,11 @@
 //
 // Measured, predictor / corrector, against one thread walking each column (64
 // columns and two warps per CTA, ten warps an SM): R2B2 L30 FP64 98 / 104 ->
-// 27 / 27 us, R2B4 L65 FP64 277 / 287 -> 205 / 220 us, R2B6 L90 double-word
+// 27 / 27 us, R2B4 L65 FP64 277 / 287 -> 197 / 213 us, R2B6 L90 double-word
 // 1.87 / 2.64 -> 1.59 / 2.06 ms, R2B5 L90 double-word over terrain 1.09 / 1.36
-// -> 0.70 / 0.94 ms.  R2B6 L90 FP64 3.41 / 3.67 -> 3.47 / 3.71 ms: there both
+// -> 0.70 / 0.94 ms.  R2B6 L90 FP64 3.41 / 3.67 -> 3.31 / 3.58 ms: there both
 // keep the FP64 unit busy (a warp's FP64 instruction takes 19 cycles of the
-// SM; 59 to 62 of them a level).
+// SM; 57 to 61 of them a level), and only the reciprocal's operations counted.
 //
 // This header holds the kernel template and its helpers; kernels_column.cu
 // instantiates the flat-ground forms (and the allocation-free entry point),
@@ -53,6 +53,7 @@
 #include <type_traits>
 
 #include "dfloat.cuh"
+#include "fp64.cuh"
 #include "kernels.h"
 
 namespace icon {
@@ -108,19 +109,6 @@ constexpr int kScratchPlanes = 8;
 // is it plus the interpolated perturbation); the explicit part
 // of the vertical pressure-gradient term is CGAM (1 - beta)/beta.
 enum { CZB = 0, CR = 1, CRN = 2, CTHI = 3, CB = 4, CGAM = 5, WG = 6, WG2 = 7 };
-
-// Reciprocal of a positive FP64 value far from the subnormal range (the
-// pivots and the equation-of-state denominator): a double-word FP32 seed
-// (about 44 correct bits, computed on the FP32 pipes) widened with one FP64
-// addition, then one Newton-Raphson step r + r (1 - x r) in FP64, which
-// squares the seed's relative error to far below double precision.  Three
-// operations on this GPU's slow FP64 pipe instead of the five of the
-// hardware approximation refined twice.
-__device__ __forceinline__ double rcp(double x) {
-  const double r = to_double(icon::rcp(to_df(x)));
-  const double e = fma(-x, r, 1.0);
-  return fma(r, e, r);
-}
 
 // 8-byte asynchronous global->shared copy (no register staging), completed
 // by cp_wait() for all copies the thread issued.

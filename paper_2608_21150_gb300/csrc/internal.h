@@ -29,7 +29,10 @@ struct GridT {
   const T* lap_c;   // [nc*3] l_e / (d_e A_c)
   const T* e2c_w;   // [nc*3] edge->cell interpolation weights
   const T* grad_c;  // [nc*6] Green-Gauss gradient in the cell frame, (x,y) per nbr: sum G_j (psi_j - psi_c)
-  const T* grad_s;  // [nc*2] sum_j G_j (x, y): the FP64 gradient as sum G_j psi_j - (sum G_j) psi_c
+  // FP64: the same gradient in the basis (G_a, G_b) of two of its three
+  // vectors, grad = G_a A + G_b B, where G_m = alpha G_a + beta G_b
+  const int* grad_nb;    // [nc*3] the neighbours a, b, m
+  const double* grad_b;  // [nc*4] alpha, beta, 1 + alpha, 1 + beta
   const T* lap_s;   // [nc]   sum_j lap_c_j (the FP64 divergence Laplacian in the same form)
   const T* e2c_wd;  // [nc*3] e2c_w times 1/d of that edge (the sum of the edges' w advection)
   const T* k4w_c;   // [nc]   hdiff_w_k4 * A_c^2
@@ -41,12 +44,14 @@ struct GridT {
   const T* f_e;     // [ne] Coriolis parameter
   const T* vt_w;    // [ne*5] tangential-wind weights: self, e2c2e[0..3]
   const T* upw;     // [ne*12] per upwind side s: (dx, dy, nx, ny, tx, ty) in that cell's frame
-  const T* upw_s;   // [ne*12] the same with n and t scaled by dt_s/2 (the back trajectory's half substep)
+  const T* upw_s;   // [ne*12] the same with n and t scaled by dt_s/2 (the back trajectory's half substep);
+                    // FP64: each pair times (G_a, G_b) of that cell, the offset seen by (A, B)
   const T* cpd_inv_d;  // [ne] cpd / d_e (the horizontal pressure gradient's factor)
-  const T* tenh_a;  // [ne] hdiff_tenh_fac A_e / dtime (enhanced temperature diffusion; null when off)
+  const T* tenh_a;  // [ne] hdiff_tenh_fac A_e / dtime (enhanced temperature diffusion; null when off; FP64: not over dtime)
   const T* nt;      // [ne*6] normal xyz, tangent xyz
   const T* inv_dn;  // [ne] 1/(arc between the two opposite diamond vertices)
   const T* smag_a;  // [ne] hdiff_smag_fac * A_e
+  const double* smag_c;  // [ne*12] FP64: |smag_a| dtime times n/d_n, t/l (tension), n/l, t/d_n (shear)
   const T* k4_a;    // [ne] hdiff_k4 * A_e^2
   const T* fdiv_e;  // [ne] divflux_fac * mean cell area / d_e (flux filter)
   const T* ddamp_e; // [ne] divdamp_fac * mean cell area^2 / d_e (divergence damping)

@@ -23,6 +23,7 @@
 #include <type_traits>
 
 #include "dfloat.cuh"
+#include "fp64.cuh"
 #include "kernels.h"
 
 namespace icon {
@@ -636,9 +637,16 @@ __global__ void __launch_bounds__(kVaThreads, 2) va_fused(GridT<float> g, VertT<
 }
 
 // -------------------------------------------------------------------------
-// A5 (predictor): Green-Gauss gradients of rho and theta_v (perturbations in
-// mixed mode: the reference is horizontally uniform) in each cell's local
-// frame: grad4 = (drho_x, drho_y, dth_x, dth_y) as 4 planes [4][nc*nlev].
+// A5 (predictor): Green-Gauss gradients of rho and theta_v as four planes
+// grad4 [4][nc*nlev].  FP64: the coefficients (A, B) of both in the cell's own
+// basis, grad = G_a A + G_b B with two of the three vectors of
+// grad = sum_j G_j (psi_j - psi_c): with G_m = alpha G_a + beta G_b,
+// A = psi_a + alpha psi_m - (1 + alpha) psi_c, two FP64 operations a component
+// where the cell frame's x and y take four, and the edge kernel's offsets are
+// stored in that basis too (upw_s).  The pair (a, b) is the least parallel one,
+// so |alpha|, |beta| <= 1 and the sums cancel no more than the frame's did.
+// 327680 cells of 90 levels: 1028 -> 619 us.  (Mixed mode: x and y of the
+// perturbations, in stencil_quad.cuh.)
 // -------------------------------------------------------------------------
 // exner_ref_c: the per-column reference exner over terrain (kTerr).
 template <bool kTerr = false>
@@ -650,27 +658,19 @@ __global__ void sn_cell_grad(GridT<double> g, VertT<double> v, const double* __r
   const int nlev = v.nlev;
   if (!flat_index(g.nc, nlev, c, k)) return;
   const size_t n = (size_t)g.nc * nlev;
-  const int* cc = g.c2e2c + 3 * (size_t)c;
-  const double* G = g.grad_c + 6 * (size_t)c;
+  const int* cc = g.grad_nb + 3 * (size_t)c;
+  const double* G = g.grad_b + 4 * (size_t)c;
   const size_t i = (size_t)c * nlev + k;
   const double ex_ref = kTerr ? exner_ref_c[i] : v.exner_ref[k];
   // extrapolated exner perturbation (1 + a) pr - a pr_old of this cell, for the
-  // pressure gradient at its edges: FP64, or a double-word pair in mixed mode
-  // (exner is near 1, the difference across an edge ~1e-5 of it)
+  // pressure gradient at its edges
   pex[i] = (1.0 + exfac) * (exner[i] - ex_ref) - exfac * exner_pr[i];
-  const size_t i0 = (size_t)cc[0] * nlev + k, i1 = (size_t)cc[1] * nlev + k, i2 = (size_t)cc[2] * nlev + k;
-  const double r = rho[i], t = theta[i];
-  // sum G_j psi_j - (sum G_j) psi_c: four FP64 operations per component
-  // instead of the differences' shared three plus three (the gradient only
-  // moves the upwind value by a small fraction of it, so the cancellation
-  // is harmless)
-  const double* S = g.grad_s + 2 * (size_t)c;
-  const double r0 = rho[i0], r1 = rho[i1], r2 = rho[i2];
-  const double t0 = theta[i0], t1 = theta[i1], t2 = theta[i2];
-  grad4[i] = fmat(G[4], r2, fmat(G[2], r1, fmat(G[0], r0, -(S[0] * r))));
-  grad4[n + i] = fmat(G[5], r2, fmat(G[3], r1, fmat(G[1], r0, -(S[1] * r))));
-  grad4[2 * n + i] = fmat(G[4], t2, fmat(G[2], t1, fmat(G[0], t0, -(S[0] * t))));
-  grad4[3 * n + i] = fmat(G[5], t2, fmat(G[3], t1, fmat(G[1], t0, -(S[1] * t))));
+  const size_t ia = (size_t)cc[0] * nlev + k, ib = (size_t)cc[1] * nlev + k, im = (size_t)cc[2] * nlev + k;
+  const double r = rho[i], rm = rho[im], t = theta[i], tm = theta[im];
+  grad4[i] = fma(G[0], rm, fma(-G[2], r, rho[ia]));
+  grad4[n + i] = fma(G[1], rm, fma(-G[3], r, rho[ib]));
+  grad4[2 * n + i] = fma(G[0], tm, fma(-G[2], t, theta[ia]));
+  grad4[3 * n + i] = fma(G[1], tm, fma(-G[3], t, theta[ib]));
 }
 
 // -------------------------------------------------------------------------
@@ -950,7 +950,10 @@ __global__ void diff_div_curl_uv(GridT<double> g, VertT<double> v, const double*
   uv3[2 * nvl + iv] = uz;
 }
 
-// edges: Smagorinsky coefficient and the vector Laplacian of vn
+// edges: Smagorinsky coefficient (times dtime) and the vector Laplacian of vn.
+// Bound by the FP64 pipe: the coefficients carry every factor of the tension
+// and the shear, and the square root takes two FP64 operations: 26 a
+// point-level instead of 35, 122880 edges of 90 levels 733 -> 554 us.
 __global__ void diff_edge_smag(GridT<double> g, VertT<double> v, const double* __restrict__ div_vn,
                                const double* __restrict__ zeta, const double* __restrict__ uv3, double* __restrict__ nu,
                                double* __restrict__ lap) {
@@ -961,20 +964,20 @@ __global__ void diff_edge_smag(GridT<double> g, VertT<double> v, const double* _
   const int* dm = g.e2c2v + 4 * (size_t)e;
   const size_t im = (size_t)dm[0] * nlev + k, ip = (size_t)dm[1] * nlev + k;
   const size_t i2 = (size_t)dm[2] * nlev + k, i3 = (size_t)dm[3] * nlev + k;
-  const double* nt = g.nt + 6 * (size_t)e;
   const double dtx = uv3[ip] - uv3[im], dty = uv3[nvl + ip] - uv3[nvl + im];
   const double dtz = uv3[2 * nvl + ip] - uv3[2 * nvl + im];
   const double dnx = uv3[i3] - uv3[i2], dny = uv3[nvl + i3] - uv3[nvl + i2];
   const double dnz = uv3[2 * nvl + i3] - uv3[2 * nvl + i2];
-  const double il = g.inv_l[e], idn = g.inv_dn[e];
+  const double* q = g.smag_c + 12 * (size_t)e;
   const double tension =
-      (dnx * nt[0] + dny * nt[1] + dnz * nt[2]) * idn - (dtx * nt[3] + dty * nt[4] + dtz * nt[5]) * il;
-  const double shear = (dtx * nt[0] + dty * nt[1] + dtz * nt[2]) * il + (dnx * nt[3] + dny * nt[4] + dnz * nt[5]) * idn;
+      fma(dnx, q[0], fma(dny, q[1], fma(dnz, q[2], -fma(dtx, q[3], fma(dty, q[4], dtz * q[5])))));
+  const double shear = fma(dtx, q[6], fma(dty, q[7], fma(dtz, q[8], fma(dnx, q[9], fma(dny, q[10], dnz * q[11])))));
   const size_t ie = (size_t)e * nlev + k;
-  nu[ie] = g.smag_a[e] * sqrt(tension * tension + shear * shear);
+  const double a = sqrt2(fma(tension, tension, shear * shear));
+  nu[ie] = g.smag_a[e] < 0.0 ? -a : a;
   const int c0 = g.e2c[2 * e], c1 = g.e2c[2 * e + 1];
   lap[ie] = (div_vn[(size_t)c1 * nlev + k] - div_vn[(size_t)c0 * nlev + k]) * g.inv_d[e] -
-            (zeta[ip] - zeta[im]) * il;
+            (zeta[ip] - zeta[im]) * g.inv_l[e];
 }
 
 // cells (half-level range): div of lap vn, cell Laplacian of w, theta increment;
@@ -1007,7 +1010,7 @@ __global__ void diff_second(GridT<double> g, VertT<double> v, ScalT<double> sc, 
         double n0 = nu[(size_t)ce[0] * nlev + k], n1 = nu[(size_t)ce[1] * nlev + k], n2 = nu[(size_t)ce[2] * nlev + k];
         if (k >= nlev - sc.tenh_levels) {
           // enhanced near-surface temperature diffusion: the edge coefficient
-          // raised by fac A_e / dtime max(e_c, e_nbr)
+          // raised by fac A_e / dtime max(e_c, e_nbr) (here all times dtime)
           const double ex = tenh_ex[ic];
           n0 += g.tenh_a[ce[0]] * max(ex, tenh_ex[(size_t)cc[0] * nlev + k]);
           n1 += g.tenh_a[ce[1]] * max(ex, tenh_ex[(size_t)cc[1] * nlev + k]);
@@ -1016,7 +1019,7 @@ __global__ void diff_second(GridT<double> g, VertT<double> v, ScalT<double> sc, 
         double f = L[0] * n0 * (theta[(size_t)cc[0] * nlev + k] - tc);
         f += L[1] * n1 * (theta[(size_t)cc[1] * nlev + k] - tc);
         f += L[2] * n2 * (theta[(size_t)cc[2] * nlev + k] - tc);
-        dtheta[ic] = sc.dtime * f;
+        dtheta[ic] = f;
       }
     }
     return;
@@ -1064,11 +1067,13 @@ __global__ void diff_edge_update(GridT<double> g, VertT<double> v, ScalT<double>
   const int vm = g.e2v[2 * e], vp = g.e2v[2 * e + 1];
   const double lap2 = (div_l[(size_t)c1 * nlev + k] - div_l[(size_t)c0 * nlev + k]) * g.inv_d[e] -
                  (curl_l[(size_t)vp * nlev + k] - curl_l[(size_t)vm * nlev + k]) * g.inv_l[e];
-  const double inc = sc.dtime * nu[ie] * lap[ie] - g.k4_a[e] * lap2;
-  vn[ie] = vn[ie] + (double)inc;
+  const double inc = nu[ie] * lap[ie] - g.k4_a[e] * lap2;
+  vn[ie] = vn[ie] + inc;
 }
 
-// cells (half-level range): w fourth-order diffusion, theta/exner update (FP64, in place)
+// cells (half-level range): w fourth-order diffusion, theta/exner update (FP64,
+// in place).  FP64 operations bound it: 12 a point-level with the reciprocal of
+// theta instead of 19 with the division, 81920 cells of 90 levels 276 -> 183 us.
 __global__ void diff_cell_update(GridT<double> g, VertT<double> v, ScalT<double> sc, double rd_o_cvd, StateView st,
                                  const double* __restrict__ lap_w, const double* __restrict__ dtheta) {
   int c, k;
@@ -1082,15 +1087,13 @@ __global__ void diff_cell_update(GridT<double> g, VertT<double> v, ScalT<double>
     l2 += L[1] * (lap_w[(size_t)cc[1] * nlevp + k] - lc);
     l2 += L[2] * (lap_w[(size_t)cc[2] * nlevp + k] - lc);
     const size_t iw = (size_t)c * nlevp + k;
-    st.w[iw] = st.w[iw] - (double)(g.k4w_c[c] * l2);
+    st.w[iw] = st.w[iw] - g.k4w_c[c] * l2;
   }
   if (k < nlev && sc.hdiff_temp) {
     const size_t ic = (size_t)c * nlev + k;
-    const double th = st.theta_v[ic];
-    const double thn = th + (double)dtheta[ic];
-    const double exn = st.exner[ic] * (1.0 + rd_o_cvd * (thn - th) / th);
-    st.theta_v[ic] = thn;
-    st.exner[ic] = exn;
+    const double th = st.theta_v[ic], dth = dtheta[ic], ex = st.exner[ic];
+    st.theta_v[ic] = th + dth;
+    st.exner[ic] = fma(ex, (rd_o_cvd * dth) * rcp(th), ex);
   }
 }
 

@@ -10,13 +10,13 @@
 // arithmetic makes of pads; no level reads them.  Every level's expression is
 // rounded as in the one-level form, so the bits are the same.
 //
-// At 81920 cells, 122880 edges and 90 levels, one level per thread -> a quad
+// At 327680 cells, 491520 edges and 90 levels, one level per thread -> a quad
 // (us a launch): va_edge_pre 197 -> 125, va_cell_vert 331 -> 179, va_edge_tend
 // 404 -> 234, va_cell_w 119 -> 71, sn_cell_grad 308 -> 238, sn_edge_pred
 // 478 -> 371, sn_cell_div 131 -> 88, sn_cell_fluxdiv 336 -> 228, mx_refresh
 // 382 -> 234, diff_div_curl_uv 262 -> 150, diff_edge_smag 402 -> 254,
 // diff_second 369 -> 241, diff_edge_update 301 -> 215, diff_cell_update
-// 405 -> 355; at 20480 cells over terrain va_concorr 80 -> 56.  DRAM bounds
+// 405 -> 355; at 81920 cells over terrain va_concorr 80 -> 56.  DRAM bounds
 // what is left; mx_refresh and the updates move the FP64 state, in pairs where
 // the caller's rows allow it.
 #pragma once
