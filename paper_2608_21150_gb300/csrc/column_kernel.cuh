@@ -362,7 +362,8 @@ __global__ void __launch_bounds__(ColForm<T, KC, CW, RL, kCorr != 0, kTerr>::NT,
   constexpr int LD = F::LD;
   extern __shared__ __align__(16) unsigned char sm_raw[];
   double* sm = reinterpret_cast<double*>(sm_raw);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned tid = after_previous(threadIdx.x);
+  const int lane = tid & 31, warp = tid >> 5;
   const int col = lane % CW;
   const int nlev = v.nlev, nlevp = nlev + 1;
   const int c0 = blockIdx.x * CW;
@@ -869,11 +870,11 @@ void launch_col_form(const Engine& en, int corrector, const ColArgs<T>& a, const
     const unsigned blocks = (unsigned)((nc + CW - 1) / CW);
     if (corrector) {
       using F = ColForm<T, KC, CW, RL, true, kTerr>;
-      ICON_LAUNCH_SMEM(name, blocks, F::NT, F::bytes, s, (sn_column<T, RA, KC, CW, RL, 1, kTerr, false>), nc, en.v,
+      ICON_CHAIN_SMEM(name, blocks, F::NT, F::bytes, s, (sn_column<T, RA, KC, CW, RL, 1, kTerr, false>), nc, en.v,
                        en.sc, 1, a);
     } else {
       using F = ColForm<T, KC, CW, RL, false, kTerr>;
-      ICON_LAUNCH_SMEM(name, blocks, F::NT, F::bytes, s, (sn_column<T, RA, KC, CW, RL, 0, kTerr, false>), nc, en.v,
+      ICON_CHAIN_SMEM(name, blocks, F::NT, F::bytes, s, (sn_column<T, RA, KC, CW, RL, 0, kTerr, false>), nc, en.v,
                        en.sc, 0, a);
     }
   });

@@ -3,6 +3,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <utility>
 #include <vector>
 
 #include "internal.h"
@@ -33,22 +34,71 @@ struct Prof {
 };
 extern thread_local Prof* g_prof;
 
-#define ICON_LAUNCH_SMEM(name, grid, block, smem, stream, kernel, ...) \
-  do {                                                                  \
-    cudaEvent_t e0_ = nullptr;                                          \
-    if (g_prof) {                                                       \
-      e0_ = g_prof->get();                                              \
-      cudaEventRecord(e0_, stream);                                     \
-    }                                                                   \
-    kernel<<<grid, block, smem, stream>>>(__VA_ARGS__);                 \
-    if (g_prof) {                                                       \
-      cudaEvent_t e1_ = g_prof->get();                                  \
-      cudaEventRecord(e1_, stream);                                     \
-      g_prof->recs.push_back({name, e0_, e1_});                         \
-    }                                                                   \
+// Kernel launches, each bracketed by an event pair when this thread profiles.
+#define ICON_LAUNCH_AS(name, stream, ...)              \
+  do {                                                 \
+    cudaEvent_t e0_ = nullptr;                         \
+    if (g_prof) {                                      \
+      e0_ = g_prof->get();                             \
+      cudaEventRecord(e0_, stream);                    \
+    }                                                  \
+    __VA_ARGS__;                                       \
+    if (g_prof) {                                      \
+      cudaEvent_t e1_ = g_prof->get();                 \
+      cudaEventRecord(e1_, stream);                    \
+      g_prof->recs.push_back({name, e0_, e1_});        \
+    }                                                  \
   } while (0)
+#define ICON_LAUNCH_SMEM(name, grid, block, smem, stream, kernel, ...) \
+  ICON_LAUNCH_AS(name, stream, kernel<<<grid, block, smem, stream>>>(__VA_ARGS__))
 #define ICON_LAUNCH(name, grid, block, stream, kernel, ...) \
   ICON_LAUNCH_SMEM(name, grid, block, 0, stream, kernel, __VA_ARGS__)
+
+// Launch with programmatic stream serialization, for kernels in which every
+// thread passes after_previous() before it touches memory that another kernel
+// writes: their CTAs are placed as soon as every CTA of the kernel before them
+// has exited, instead of after its writes are flushed and the launch is
+// processed.
+//
+// A step is a chain of 70 to 100 dependent launches, 2-6 us each on a small
+// grid.  Plain launches -> these, us: the mixed substep of R2B3 L31 136 -> 95,
+// the FP64 step of R2B2 L30 444 -> 425 and of R2B4 L65 4761 -> 4744, the
+// learned step of R2B5 L90 6716 -> 6687, four training steps of 4096 rows
+// 1246 -> 1121.  An explicit trigger in the kernels (the next one's CTAs then
+// wait resident, beside the running ones) lost: 568 at R2B2 with the trigger
+// behind the wait, 839 with it in front, and 35.4 ms instead of 32.7 for the
+// mixed step of R2B6.
+template <class... P, class... A>
+void launch_chained(unsigned grid, unsigned block, size_t smem, cudaStream_t s, void (*kernel)(P...), A&&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = g_prof ? 0 : 1;  // a timed launch runs alone
+  cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+#define ICON_CHAIN_SMEM(name, grid, block, smem, stream, kernel, ...) \
+  ICON_LAUNCH_AS(name, stream, launch_chained(grid, block, smem, stream, kernel, __VA_ARGS__))
+#define ICON_CHAIN(name, grid, block, stream, kernel, ...) \
+  ICON_CHAIN_SMEM(name, grid, block, 0, stream, kernel, __VA_ARGS__)
+
+// x, once the kernels before this one on its stream are complete and their
+// writes are visible.  Every thread calls it, those without work too: a kernel
+// is then complete only after its predecessor, so the one after it sees both.
+// Indices that lead to memory are made from the result, so that no load can be
+// moved ahead of the wait.
+__device__ __forceinline__ unsigned after_previous(unsigned x) {
+#ifdef __CUDA_ARCH__
+  asm volatile("griddepcontrol.wait;" : "+r"(x)::"memory");
+#endif
+  return x;
+}
+__device__ __forceinline__ unsigned flat_thread() { return after_previous(blockIdx.x * blockDim.x + threadIdx.x); }
 
 // Device pointers of one prognostic state (level-contiguous, FP64).
 struct StateView {

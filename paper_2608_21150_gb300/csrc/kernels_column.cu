@@ -327,16 +327,16 @@ extern "C" int icon_column_solve_noalloc(int32_t n_cols, int32_t nlev, const dou
     using F = NoallocNarrow;
     const unsigned blocks = (unsigned)((n_cols + kColNarrow - 1) / kColNarrow);
     if (dw)
-      sn_column<double, dws, 8, kColNarrow, 1, -1, false, true><<<blocks, F::NT, F::bytes, stream>>>(n_cols, v, s, corrector, a);
+      launch_chained(blocks, F::NT, F::bytes, stream, sn_column<double, dws, 8, kColNarrow, 1, -1, false, true>, n_cols, v, s, corrector, a);
     else
-      sn_column<double, double, 8, kColNarrow, 1, -1, false, true><<<blocks, F::NT, F::bytes, stream>>>(n_cols, v, s, corrector, a);
+      launch_chained(blocks, F::NT, F::bytes, stream, sn_column<double, double, 8, kColNarrow, 1, -1, false, true>, n_cols, v, s, corrector, a);
   } else {
     using F = NoallocWide;
     const unsigned blocks = (unsigned)((n_cols + kColWide - 1) / kColWide);
     if (dw)
-      sn_column<double, dws, 8, kColWide, 2, -1, false, true><<<blocks, F::NT, F::bytes, stream>>>(n_cols, v, s, corrector, a);
+      launch_chained(blocks, F::NT, F::bytes, stream, sn_column<double, dws, 8, kColWide, 2, -1, false, true>, n_cols, v, s, corrector, a);
     else
-      sn_column<double, double, 8, kColWide, 2, -1, false, true><<<blocks, F::NT, F::bytes, stream>>>(n_cols, v, s, corrector, a);
+      launch_chained(blocks, F::NT, F::bytes, stream, sn_column<double, double, 8, kColWide, 2, -1, false, true>, n_cols, v, s, corrector, a);
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return report_error(ICON_ERR_CUDA, std::string(fn) + cudaGetErrorString(e));

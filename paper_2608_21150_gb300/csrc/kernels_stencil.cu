@@ -42,11 +42,10 @@ __device__ __forceinline__ double f2d(float x) { return f2d_exact(x); }
 __device__ __forceinline__ float d2f(double x) { return to_float(to_df(x)); }
 
 __device__ __forceinline__ bool flat_index(int n_h, int nk, int& h, int& k) {
-  unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (unsigned)n_h * (unsigned)nk) return false;
-  h = (int)(i / (unsigned)nk);
-  k = (int)(i - (unsigned)h * (unsigned)nk);
-  return true;
+  const unsigned i = blockIdx.x * blockDim.x + threadIdx.x, q = i / (unsigned)nk;
+  k = (int)(i - q * (unsigned)nk);
+  h = (int)after_previous(q);
+  return i < (unsigned)n_h * (unsigned)nk;
 }
 
 inline unsigned blocks_for(long long n, int threads) { return (unsigned)((n + threads - 1) / threads); }
@@ -60,7 +59,9 @@ __device__ __forceinline__ float fmat(float a, float b, float c) { return fmaf(a
 // point's neighbour indices and weights are loaded once per warp.  The default
 // of the FP32 sn_edge_corr; not of the FP64 kernels, where 90 levels fill only
 // 90 of 96 lane slots of the saturated FP64 pipe (the tuner tries both).
-__device__ __forceinline__ int warp_point() { return (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); }
+__device__ __forceinline__ int warp_point() {
+  return (int)after_previous(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
+}
 __device__ __forceinline__ int lane_id() { return (int)(threadIdx.x & 31u); }
 inline unsigned blocks_for_points(long long n_points, int threads) {
   const int warps = threads / 32;
@@ -198,7 +199,7 @@ __global__ void va_cell_vert(GridT<double> g, VertT<double> v, const double* __r
                              double* __restrict__ zeta, double* __restrict__ w_v, double* __restrict__ wq,
                              const double* __restrict__ wcc) {
   const int nlev = v.nlev, nlevp = nlev + 1;
-  unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned i = flat_thread();
   const unsigned ncell = (unsigned)g.nc * nlev;
   if (i < ncell) {
     int c = (int)(i / (unsigned)nlev), k = (int)(i - (unsigned)c * nlev);
@@ -393,7 +394,7 @@ __global__ void __launch_bounds__(kVaThreads, 2) va_fused(GridT<float> g, VertT<
                                                           float* __restrict__ divd2) {
   extern __shared__ float sf[];
   constexpr int L = kVaL, S = kVaS, Sn = kVaSn;
-  const int p = blockIdx.x;
+  const int p = (int)after_previous(blockIdx.x);
   const int nlev = v.nlev, ld = v.ldf;
   const int e0a = pt.off_e0[p], ne0 = pt.off_e0[p + 1] - e0a;
   const int e1a = pt.off_e1[p], ne1 = pt.off_e1[p + 1] - e1a;
@@ -743,7 +744,7 @@ __global__ void sn_edge_hpg_steep(GridT<T> g, VertT<T> v, ScalT<T> sc, int n, co
                                   const double* __restrict__ exref_c, const double* __restrict__ cid64,
                                   const T* __restrict__ theta_e, const T* __restrict__ vn,
                                   const T* __restrict__ ddt_vn, T* __restrict__ hpg, T* __restrict__ vn_p) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = (int)flat_thread();
   if (i >= n) return;
   const int nlev = v.nlev, ldf = v.ldf;
   const int e = idx[4 * i], k = idx[4 * i + 1];
@@ -917,7 +918,7 @@ __global__ void sn_cell_fluxsum(GridT<double> g, VertT<double> v, const double* 
 __global__ void diff_div_curl_uv(GridT<double> g, VertT<double> v, const double* __restrict__ vn,
                                  double* __restrict__ div_vn, double* __restrict__ zeta, double* __restrict__ uv3) {
   const int nlev = v.nlev;
-  unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned i = flat_thread();
   const unsigned ncell = (unsigned)g.nc * nlev;
   if (i < ncell) {
     int c = (int)(i / (unsigned)nlev), k = (int)(i - (unsigned)c * nlev);
@@ -988,7 +989,7 @@ __global__ void diff_second(GridT<double> g, VertT<double> v, ScalT<double> sc, 
                             double* __restrict__ dtheta, double* __restrict__ curl_l,
                             const double* __restrict__ tenh_ex) {
   const int nlev = v.nlev, nlevp = nlev + 1;
-  unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned i = flat_thread();
   const unsigned ncell = (unsigned)g.nc * nlevp;
   if (i < ncell) {
     int c = (int)(i / (unsigned)nlevp), k = (int)(i - (unsigned)c * nlevp);
@@ -1044,7 +1045,7 @@ template <class T>
 __global__ void diff_tenh_excess(GridT<T> g, VertT<T> v, ScalT<T> sc, const T* __restrict__ theta,
                                  T* __restrict__ ex) {
   const int nlev = v.nlev, ldf = v.ldf, nl = sc.tenh_levels;
-  const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned i = flat_thread();
   if (i >= (unsigned)g.nc * (unsigned)nl) return;
   const int c = (int)(i / (unsigned)nl), k = nlev - nl + (int)(i - (unsigned)c * (unsigned)nl);
   const int* cc = g.c2e2c + 3 * (size_t)c;
@@ -1125,44 +1126,44 @@ void launch_velocity_tendencies(const Ctx<T>& x, const T* vn, const T* w, T* ddt
       const VaPatchT& pt = x.vp;
       const size_t smem =
           va_fused_smem_floats(pt.max_e0, pt.max_e1, pt.max_c3, pt.max_c0, pt.max_v3, pt.max_e4) * sizeof(float);
-      ICON_LAUNCH_SMEM("va_fused_f32", (unsigned)pt.n_patches, kVaThreads, smem, s, va_fused, g, v, pt, vn, w, wk.vt,
+      ICON_CHAIN_SMEM("va_fused_f32", (unsigned)pt.n_patches, kVaThreads, smem, s, va_fused, g, v, pt, vn, w, wk.vt,
                        ddt_vn, ddt_w, divd, divd2);
       return;
     }
     // four levels per thread
     const long long nqf = quads_full(nlev), nqh = quads_half(nlev);
     T* const q_wcc = terr ? wcc : nullptr;
-    ICON_LAUNCH("va_edge_pre_f32", blocks_for(g.ne * nqf, TH(0)), TH(0), s, va_edge_pre_q, g, v, vn, wk.vt, wk.ekin_e,
+    ICON_CHAIN("va_edge_pre_f32", blocks_for(g.ne * nqf, TH(0)), TH(0), s, va_edge_pre_q, g, v, vn, wk.vt, wk.ekin_e,
                 wk.vn_ie, terr ? tr.wgt_e : nullptr);
     if (terr)
-      ICON_LAUNCH("va_concorr_f32", blocks_for(g.nc * nqh, TH(14)), TH(14), s, va_concorr_q, g, v, tr, wk.vn_ie,
+      ICON_CHAIN("va_concorr_f32", blocks_for(g.nc * nqh, TH(14)), TH(14), s, va_concorr_q, g, v, tr, wk.vn_ie,
                   wk.vt, wcc);
-    ICON_LAUNCH("va_cell_vert_f32", blocks_for(g.nc * nqf + g.nv * nqh, TH(1)), TH(1), s, va_cell_vert_q, g, v, vn, w,
+    ICON_CHAIN("va_cell_vert_f32", blocks_for(g.nc * nqf + g.nv * nqh, TH(1)), TH(1), s, va_cell_vert_q, g, v, vn, w,
                 wk.ekin_e, wk.ekin_c, divd, divd2, wk.zeta, wk.w_v, wk.wq, q_wcc);
     const char* const nm_tend = terr ? "va_edge_tend_terrain_f32" : "va_edge_tend_f32";
     const char* const nm_w = terr ? "va_cell_w_terrain_f32" : "va_cell_w_f32";
-    ICON_LAUNCH(nm_tend, blocks_for(g.ne * nqh, TH(2)), TH(2), s, (terr ? va_edge_tend_q<true> : va_edge_tend_q<false>),
+    ICON_CHAIN(nm_tend, blocks_for(g.ne * nqh, TH(2)), TH(2), s, (terr ? va_edge_tend_q<true> : va_edge_tend_q<false>),
                 g, v, wk.vn_ie, w, wk.vt, wk.ekin_c, wk.zeta, wk.w_v, ddt_vn, wk.gw_e, tr, wk.wq);
-    ICON_LAUNCH(nm_w, blocks_for(g.nc * nqh, TH(3)), TH(3), s, (terr ? va_cell_w_q<true> : va_cell_w_q<false>), g, v,
+    ICON_CHAIN(nm_w, blocks_for(g.nc * nqh, TH(3)), TH(3), s, (terr ? va_cell_w_q<true> : va_cell_w_q<false>), g, v,
                 w, wk.gw_e, ddt_w, tr, q_wcc);
   } else {
-    ICON_LAUNCH("va_edge_pre", blocks_by_shape(SH(0), g.ne, nlev, TH(0)), TH(0), s, va_edge_pre, g, v, vn, wk.vt,
+    ICON_CHAIN("va_edge_pre", blocks_by_shape(SH(0), g.ne, nlev, TH(0)), TH(0), s, va_edge_pre, g, v, vn, wk.vt,
                 wk.ekin_e, wk.vn_ie, terr ? tr.wgt_e : nullptr, SH(0));
     if (terr)
-      ICON_LAUNCH("va_concorr", blocks_for((long long)g.nc * nlevp, TH(14)), TH(14), s, va_concorr, g, v, tr,
+      ICON_CHAIN("va_concorr", blocks_for((long long)g.nc * nlevp, TH(14)), TH(14), s, va_concorr, g, v, tr,
                   wk.vn_ie, wk.vt, wcc);
     const long long n2 = (long long)g.nc * nlev + (long long)g.nv * nlevp;
-    ICON_LAUNCH("va_cell_vert", blocks_for(n2, TH(1)), TH(1), s, va_cell_vert, g, v, vn, w, wk.ekin_e, wk.ekin_c, divd,
+    ICON_CHAIN("va_cell_vert", blocks_for(n2, TH(1)), TH(1), s, va_cell_vert, g, v, vn, w, wk.ekin_e, wk.ekin_c, divd,
                 divd2, wk.zeta, wk.w_v, wk.wq, terr ? (const T*)wcc : nullptr);
     if (terr) {
-      ICON_LAUNCH("va_edge_tend_terrain", blocks_for((long long)g.ne * nlevp, TH(2)), TH(2), s, va_edge_tend<true>, g,
+      ICON_CHAIN("va_edge_tend_terrain", blocks_for((long long)g.ne * nlevp, TH(2)), TH(2), s, va_edge_tend<true>, g,
                   v, wk.vn_ie, w, wk.vt, wk.ekin_c, wk.zeta, wk.w_v, ddt_vn, wk.gw_e, tr, (const T*)wk.wq);
-      ICON_LAUNCH("va_cell_w_terrain", blocks_by_shape(SH(3), g.nc, nlevp, TH(3)), TH(3), s, va_cell_w<true>, g, v, w,
+      ICON_CHAIN("va_cell_w_terrain", blocks_by_shape(SH(3), g.nc, nlevp, TH(3)), TH(3), s, va_cell_w<true>, g, v, w,
                   wk.gw_e, ddt_w, tr, wcc, SH(3));
     } else {
-      ICON_LAUNCH("va_edge_tend", blocks_for((long long)g.ne * nlevp, TH(2)), TH(2), s, va_edge_tend<false>, g, v,
+      ICON_CHAIN("va_edge_tend", blocks_for((long long)g.ne * nlevp, TH(2)), TH(2), s, va_edge_tend<false>, g, v,
                   wk.vn_ie, w, wk.vt, wk.ekin_c, wk.zeta, wk.w_v, ddt_vn, wk.gw_e, tr, (const T*)wk.wq);
-      ICON_LAUNCH("va_cell_w", blocks_by_shape(SH(3), g.nc, nlevp, TH(3)), TH(3), s, va_cell_w<false>, g, v, w,
+      ICON_CHAIN("va_cell_w", blocks_by_shape(SH(3), g.nc, nlevp, TH(3)), TH(3), s, va_cell_w<false>, g, v, w,
                   wk.gw_e, ddt_w, tr, wcc, SH(3));
     }
   }
@@ -1179,13 +1180,13 @@ void launch_fluxdiv(const Engine& en, const Ctx<T>& x, const T* vn, const char* 
   const WorkT<T>& wk = x.w;
   const int nlev = v.nlev;
   if constexpr (kMixed<T>) {
-    ICON_LAUNCH(name, blocks_for((long long)g.nc * quads_full(nlev), TH(7)), TH(7), s, sn_cell_fluxdiv_q<kTerr>, g, v,
+    ICON_CHAIN(name, blocks_for((long long)g.nc * quads_full(nlev), TH(7)), TH(7), s, sn_cell_fluxdiv_q<kTerr>, g, v,
                 vn, wk.divd, wk.rho_e, wk.theta_e, reinterpret_cast<df*>(en.wk.div_m),
                 reinterpret_cast<df*>(en.wk.div_t), x.tr.fx_ratio);
   } else {
-    ICON_LAUNCH("sn_edge_flux", blocks_for((long long)g.ne * nlev, TH(15)), TH(15), s, sn_edge_flux, g, v, vn,
+    ICON_CHAIN("sn_edge_flux", blocks_for((long long)g.ne * nlev, TH(15)), TH(15), s, sn_edge_flux, g, v, vn,
                 wk.divd, wk.rho_e, wk.theta_e, wk.flx_m, wk.flx_t);
-    ICON_LAUNCH(kTerr ? "sn_cell_fluxsum_terrain" : "sn_cell_fluxsum", blocks_for((long long)g.nc * nlev, TH(7)),
+    ICON_CHAIN(kTerr ? "sn_cell_fluxsum_terrain" : "sn_cell_fluxsum", blocks_for((long long)g.nc * nlev, TH(7)),
                 TH(7), s, (sn_cell_fluxsum<kTerr>), g, v, wk.flx_m, wk.flx_t, en.wk.div_m, en.wk.div_t,
                 x.tr.fx_ratio);
   }
@@ -1241,28 +1242,28 @@ void substep_impl(const Engine& en, const Ctx<T>& x, const StateView& st, cudaSt
                                 kTerr ? tr.wcc0 : nullptr, shapes);
   if (en.io_wait) stream_wait_io(s, en.io_wait);  // rho, theta_v, exner, exner_pr from here on
   if constexpr (kMixed<T>) {
-    ICON_LAUNCH(nm_grad, blocks_for(g.nc * nqf, TH(4)), TH(4), s, sn_cell_grad_q<kTerr>, g, v, s_rho, s_th, wk.grad4,
+    ICON_CHAIN(nm_grad, blocks_for(g.nc * nqf, TH(4)), TH(4), s, sn_cell_grad_q<kTerr>, g, v, s_rho, s_th, wk.grad4,
                 st.exner, st.exner_pr, en.sc.exfac, reinterpret_cast<df*>(en.wk.pex), ex_ref_c, pairs);
-    ICON_LAUNCH(nm_pred, blocks_for(g.ne * nqf, TH(5)), TH(5), s, sn_edge_pred_q<kTerr>, g, v, x.s, s_vn, wk.vt,
+    ICON_CHAIN(nm_pred, blocks_for(g.ne * nqf, TH(5)), TH(5), s, sn_edge_pred_q<kTerr>, g, v, x.s, s_vn, wk.vt,
                 wk.ddt_vn0, s_rho, s_th, reinterpret_cast<const df*>(en.wk.pex), wk.grad4, wk.rho_e, wk.theta_e,
                 wk.hpg, wk.vn_p, tr);
   } else {
-    ICON_LAUNCH(nm_grad, blocks_for(nce, TH(4)), TH(4), s, sn_cell_grad<kTerr>, g, v, s_rho, s_th, wk.grad4, st.exner,
+    ICON_CHAIN(nm_grad, blocks_for(nce, TH(4)), TH(4), s, sn_cell_grad<kTerr>, g, v, s_rho, s_th, wk.grad4, st.exner,
                 st.exner_pr, en.sc.exfac, en.wk.pex, ex_ref_c);
-    ICON_LAUNCH(nm_pred, blocks_for(nee, TH(5)), TH(5), s, sn_edge_pred<kTerr>, g, v, x.s, s_vn, wk.vt, wk.ddt_vn0,
+    ICON_CHAIN(nm_pred, blocks_for(nee, TH(5)), TH(5), s, sn_edge_pred<kTerr>, g, v, x.s, s_vn, wk.vt, wk.ddt_vn0,
                 s_rho, s_th, en.wk.pex, en.g64.cpd_inv_d, wk.grad4, wk.rho_e, wk.theta_e, wk.hpg, wk.vn_p, tr);
   }
   if (kTerr && en.v.n_steep > 0)
-    ICON_LAUNCH(kname<T>("sn_edge_hpg_steep", "sn_edge_hpg_steep_f32"), blocks_for(en.v.n_steep, 128), 128, s,
+    ICON_CHAIN(kname<T>("sn_edge_hpg_steep", "sn_edge_hpg_steep_f32"), blocks_for(en.v.n_steep, 128), 128, s,
                 sn_edge_hpg_steep<T>, g, v, x.s, en.v.n_steep, en.v.steep_idx, en.v.steep_w, en.wk.pex,
                 en.v.exner_ref_c, en.g64.cpd_inv_d, wk.theta_e, s_vn, wk.ddt_vn0, wk.hpg, wk.vn_p);
   // divergence of a velocity field; the predictor's call also updates the exner history
   auto cell_div = [&](const T* vn, double* exner_pr) {
     if constexpr (kMixed<T>)
-      ICON_LAUNCH(nm_div, blocks_for(g.nc * nqf, TH(6)), TH(6), s, sn_cell_div_q<kTerr>, g, v, vn, wk.divd, st.exner,
+      ICON_CHAIN(nm_div, blocks_for(g.nc * nqf, TH(6)), TH(6), s, sn_cell_div_q<kTerr>, g, v, vn, wk.divd, st.exner,
                   exner_pr, ex_ref_c, pairs);
     else
-      ICON_LAUNCH(nm_div, blocks_by_shape(SH(6), g.nc, nlev, TH(6)), TH(6), s, sn_cell_div<kTerr>, g, v, vn, wk.divd,
+      ICON_CHAIN(nm_div, blocks_by_shape(SH(6), g.nc, nlev, TH(6)), TH(6), s, sn_cell_div<kTerr>, g, v, vn, wk.divd,
                   st.exner, exner_pr, ex_ref_c, SH(6));
   };
   cell_div(wk.vn_p, st.exner_pr);
@@ -1274,7 +1275,7 @@ void substep_impl(const Engine& en, const Ctx<T>& x, const StateView& st, cudaSt
   // ---------------- corrector ----------------
   launch_velocity_tendencies<T>(x, wk.vn_p, s_wp, wk.ddt_vn1, wk.ddt_w1, wk.divd, wk.divd2, s, threads,
                                 kTerr ? tr.wcc1 : nullptr, shapes);
-  ICON_LAUNCH(kname<T>("sn_edge_corr", "sn_edge_corr_f32"), blocks_by_shape(SH(8), g.ne, nlev, TH(8)), TH(8), s,
+  ICON_CHAIN(kname<T>("sn_edge_corr", "sn_edge_corr_f32"), blocks_by_shape(SH(8), g.ne, nlev, TH(8)), TH(8), s,
               sn_edge_corr<T>, g, v, x.s, st.vn, wk.ddt_vn0, wk.ddt_vn1, wk.hpg, wk.divd2, m.vn, SH(8));
   const T* vn_new = kMixed<T> ? (const T*)m.vn : (const T*)st.vn;
   cell_div(vn_new, nullptr);
@@ -1311,34 +1312,34 @@ void launch_diffusion(const Engine& en, const Ctx<T>& x, const StateView& st, cu
   const long long n1 = (long long)(g.nc + g.nv) * nlev;
   const long long n3 = (long long)g.nc * nlevp + (long long)g.nv * nlev;
   if constexpr (kMixed<T>) {  // four levels per thread
-    ICON_LAUNCH("diff_div_curl_uv_f32", blocks_for((g.nc + g.nv) * nqf, TH(9)), TH(9), s, diff_div_curl_uv_q, g, v,
+    ICON_CHAIN("diff_div_curl_uv_f32", blocks_for((g.nc + g.nv) * nqf, TH(9)), TH(9), s, diff_div_curl_uv_q, g, v,
                 s_vn, wk.div_vn, wk.zeta, wk.uv3);
-    ICON_LAUNCH("diff_edge_smag_f32", blocks_for(g.ne * nqf, TH(10)), TH(10), s, diff_edge_smag_q, g, v, wk.div_vn,
+    ICON_CHAIN("diff_edge_smag_f32", blocks_for(g.ne * nqf, TH(10)), TH(10), s, diff_edge_smag_q, g, v, wk.div_vn,
                 wk.zeta, wk.uv3, wk.nu, wk.lap_vn);
   } else {
-    ICON_LAUNCH("diff_div_curl_uv", blocks_for(n1, TH(9)), TH(9), s, diff_div_curl_uv, g, v, s_vn, wk.div_vn, wk.zeta,
+    ICON_CHAIN("diff_div_curl_uv", blocks_for(n1, TH(9)), TH(9), s, diff_div_curl_uv, g, v, s_vn, wk.div_vn, wk.zeta,
                 wk.uv3);
-    ICON_LAUNCH("diff_edge_smag", blocks_for((long long)g.ne * nlev, TH(10)), TH(10), s, diff_edge_smag, g, v,
+    ICON_CHAIN("diff_edge_smag", blocks_for((long long)g.ne * nlev, TH(10)), TH(10), s, diff_edge_smag, g, v,
                 wk.div_vn, wk.zeta, wk.uv3, wk.nu, wk.lap_vn);
   }
   if (x.s.tenh_levels > 0 && x.s.hdiff_temp)
-    ICON_LAUNCH(kname<T>("diff_tenh_excess", "diff_tenh_excess_f32"),
+    ICON_CHAIN(kname<T>("diff_tenh_excess", "diff_tenh_excess_f32"),
                 blocks_for((long long)g.nc * x.s.tenh_levels, kThreads), kThreads, s, diff_tenh_excess<T>, g, v, x.s,
                 s_th, wk.tenh_ex);
   if constexpr (kMixed<T>) {
-    ICON_LAUNCH("diff_second_f32", blocks_for(g.nc * nqh + g.nv * nqf, TH(11)), TH(11), s, diff_second_q, g, v, x.s,
+    ICON_CHAIN("diff_second_f32", blocks_for(g.nc * nqh + g.nv * nqf, TH(11)), TH(11), s, diff_second_q, g, v, x.s,
                 wk.lap_vn, wk.nu, s_w, s_th, wk.div_l, wk.lap_w, wk.dtheta, wk.curl_l, wk.tenh_ex);
-    ICON_LAUNCH("diff_edge_update_f32", blocks_for(g.ne * nqf, TH(12)), TH(12), s, diff_edge_update_q, g, v, x.s,
+    ICON_CHAIN("diff_edge_update_f32", blocks_for(g.ne * nqf, TH(12)), TH(12), s, diff_edge_update_q, g, v, x.s,
                 st.vn, wk.nu, wk.lap_vn, wk.div_l, wk.curl_l, m.vn, aligned_pairs(nlev, {st.vn}));
-    ICON_LAUNCH("diff_cell_update_f32", blocks_for(g.nc * nqh, TH(13)), TH(13), s, diff_cell_update_q, g, v, x.s,
+    ICON_CHAIN("diff_cell_update_f32", blocks_for(g.nc * nqh, TH(13)), TH(13), s, diff_cell_update_q, g, v, x.s,
                 en.v.theta_ref, en.sc.rd_o_cvd, st, wk.lap_w, wk.dtheta, m,
                 aligned_pairs(nlev, {st.theta_v, st.exner}));
   } else {
-    ICON_LAUNCH("diff_second", blocks_for(n3, TH(11)), TH(11), s, diff_second, g, v, x.s, wk.lap_vn, wk.nu, s_w, s_th,
+    ICON_CHAIN("diff_second", blocks_for(n3, TH(11)), TH(11), s, diff_second, g, v, x.s, wk.lap_vn, wk.nu, s_w, s_th,
                 wk.div_l, wk.lap_w, wk.dtheta, wk.curl_l, wk.tenh_ex);
-    ICON_LAUNCH("diff_edge_update", blocks_for((long long)g.ne * nlev, TH(12)), TH(12), s, diff_edge_update, g, v,
+    ICON_CHAIN("diff_edge_update", blocks_for((long long)g.ne * nlev, TH(12)), TH(12), s, diff_edge_update, g, v,
                 x.s, st.vn, wk.nu, wk.lap_vn, wk.div_l, wk.curl_l);
-    ICON_LAUNCH("diff_cell_update", blocks_for((long long)g.nc * nlevp, TH(13)), TH(13), s, diff_cell_update, g, v,
+    ICON_CHAIN("diff_cell_update", blocks_for((long long)g.nc * nlevp, TH(13)), TH(13), s, diff_cell_update, g, v,
                 x.s, en.sc.rd_o_cvd, st, wk.lap_w, wk.dtheta);
   }
 }
@@ -1368,7 +1369,7 @@ const char* const kStencilNames[kNumStencils] = {
 void launch_refresh_mirrors(const Engine& en, const StateView& st, cudaStream_t s) {
   const int nlev = en.v.nlev;
   const long long n = (long long)en.g64.ne * quads_full(nlev) + (long long)en.g64.nc * quads_half(nlev);
-  ICON_LAUNCH("mx_refresh", blocks_for(n, kThreads), kThreads, s, mx_refresh, en.g64.ne, en.g64.nc, en.c32.v,
+  ICON_CHAIN("mx_refresh", blocks_for(n, kThreads), kThreads, s, mx_refresh, en.g64.ne, en.g64.nc, en.c32.v,
               en.v.theta_ref, en.rho_ref64, st, en.m, aligned_pairs(nlev, {st.vn, st.rho, st.theta_v}));
 }
 

@@ -99,7 +99,7 @@ __global__ void va_cell_vert_q(GridT<float> g, VertT<float> v, const float* __re
                                float* __restrict__ zeta, float* __restrict__ w_v, float* __restrict__ wq,
                                const float* __restrict__ wcc) {
   const int nlev = v.nlev, ld = v.ldf, nqf = quads_full(nlev), nqh = quads_half(nlev);
-  unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned t = flat_thread();
   const unsigned ncell = (unsigned)g.nc * nqf;
   if (t < ncell) {
     const int c = (int)(t / (unsigned)nqf), k = 4 * (int)(t - (unsigned)c * nqf);
@@ -628,7 +628,7 @@ __device__ __forceinline__ void st4(double* p, const double (&a)[4], int k, int 
 __global__ void mx_refresh(int ne, int nc, VertT<float> v, const double* __restrict__ theta_ref,
                            const double* __restrict__ rho_ref, StateView st, Mirrors m, bool pairs) {
   const int nlev = v.nlev, ld = v.ldf, nqf = quads_full(nlev), nqh = quads_half(nlev);
-  unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned t = flat_thread();
   const unsigned nedge = (unsigned)ne * nqf;
   double x[4] = {}, y[4] = {};
   float o[4];
@@ -663,7 +663,7 @@ __global__ void mx_refresh(int ne, int nc, VertT<float> v, const double* __restr
 __global__ void diff_div_curl_uv_q(GridT<float> g, VertT<float> v, const float* __restrict__ vn,
                                    float* __restrict__ div_vn, float* __restrict__ zeta, float* __restrict__ uv3) {
   const int nlev = v.nlev, ld = v.ldf, nq = quads_full(nlev);
-  unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned t = flat_thread();
   const unsigned ncell = (unsigned)g.nc * nq;
   if (t < ncell) {
     const int c = (int)(t / (unsigned)nq), k = 4 * (int)(t - (unsigned)c * nq);
@@ -767,7 +767,7 @@ __global__ void diff_second_q(GridT<float> g, VertT<float> v, ScalT<float> sc, c
                               float* __restrict__ dtheta, float* __restrict__ curl_l,
                               const float* __restrict__ tenh_ex) {
   const int nlev = v.nlev, ld = v.ldf, nqf = quads_full(nlev), nqh = quads_half(nlev);
-  unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned t = flat_thread();
   const unsigned ncell = (unsigned)g.nc * nqh;
   if (t < ncell) {
     const int c = (int)(t / (unsigned)nqh), k = 4 * (int)(t - (unsigned)c * nqh);
