@@ -291,11 +291,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc(const __grid_constant__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  const int tile0 = (int)after_previous(blockIdx.x);  // the barriers and TMEM are ready before the operands are
 
   int issued = 0;  // k-blocks whose TMA loads the producer lane issued (all tiles)
   if (warp == 0 && lane == 0) {
     int g = 0;
-    for (int tile = blockIdx.x; tile < n_tiles && !*abort_flag; tile += gridDim.x) {
+    for (int tile = tile0; tile < n_tiles && !*abort_flag; tile += gridDim.x) {
       const int m0 = (tile / tiles_n) * TBM, n0 = (tile % tiles_n) * TBN;
       for (int kb = 0; kb < nk; ++kb, ++g) {
         const int s = g % kStages;
@@ -310,7 +311,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc(const __grid_constant__
     constexpr uint32_t idesc = idesc_bf16(TBM, TBN);
     int g = 0, t = 0;
     bool ok = true;
-    for (int tile = blockIdx.x; ok && tile < n_tiles; tile += gridDim.x, ++t) {
+    for (int tile = tile0; ok && tile < n_tiles; tile += gridDim.x, ++t) {
       const int b = t & 1;
       const uint32_t d = tmem + (uint32_t)(b * TBN);
       if (t >= 2 && !mbar_wait(&acc_empty[b], ((t >> 1) & 1) ^ 1, abort_flag)) break;
@@ -342,7 +343,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc(const __grid_constant__
     // half of the columns
     const int quarter = warp & 3, half = (warp - 2) >> 2;
     int t = 0;
-    for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++t) {
+    for (int tile = tile0; tile < n_tiles; tile += gridDim.x, ++t) {
       const int b = t & 1;
       // warp-uniform decision: the tcgen05.ld below is a warp-collective instruction
       if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[b], (t >> 1) & 1, abort_flag))) break;
@@ -491,7 +492,7 @@ __device__ __forceinline__ void cp16(void* smem, const void* g) {
 }
 __global__ void __launch_bounds__(kPrepThreads) layer_prep(PrepArgs a) {
   __shared__ __align__(16) unsigned char raw[kSumStages * kSumRows * 32 * sizeof(float)];
-  const int tid = threadIdx.x, nsum = (a.cols + 31) / 32;
+  const int tid = (int)after_previous(threadIdx.x), nsum = (a.cols + 31) / 32;
   int bid = blockIdx.x;
   if (bid < nsum) {
     auto tile = reinterpret_cast<float(*)[kSumRows][32]>(raw);
@@ -562,7 +563,7 @@ constexpr int kRowWarps = 8;
 __global__ void gelu_backward(int rows, int cols, const float* __restrict__ dh, int ldd,
                               const float* __restrict__ z, int ldz, float* __restrict__ dz32,
                               __nv_bfloat16* __restrict__ dz16, int ldo) {
-  const int r = blockIdx.x * kRowWarps + (threadIdx.x >> 5);
+  const int r = (int)after_previous(blockIdx.x * kRowWarps + (threadIdx.x >> 5));
   if (r >= rows) return;
 #pragma unroll 4
   for (int c = threadIdx.x & 31; c < cols; c += 32) {
@@ -575,7 +576,7 @@ __global__ void gelu_backward(int rows, int cols, const float* __restrict__ dh, 
 // fp32 -> bf16 copy with padding (pads written as zero)
 __global__ void to_bf16(int rows, int cols, const float* __restrict__ in, int ldi, __nv_bfloat16* __restrict__ out,
                         int ldo) {
-  const int r = blockIdx.x * kRowWarps + (threadIdx.x >> 5);
+  const int r = (int)after_previous(blockIdx.x * kRowWarps + (threadIdx.x >> 5));
   if (r >= rows) return;
 #pragma unroll 4
   for (int c = threadIdx.x & 31; c < ldo; c += 32)
@@ -597,17 +598,18 @@ __device__ __forceinline__ float adam_value(const AdamScal& q, float w, float gi
 }
 __global__ void __launch_bounds__(256) adam_update(AdamLayers ly, AdamScal q) {
   __shared__ __nv_bfloat16 tile[32][34];
+  const int tid = (int)after_previous(threadIdx.x);
   int l = 0;
   while (l < 2 && (int)blockIdx.x >= ly.l[l].block_end) ++l;
   const AdamLayer& a = ly.l[l];
   const int bid = (int)blockIdx.x - (l ? ly.l[l - 1].block_end : 0);
   const int tk = (a.n_in + 31) / 32, nt = tk * ((a.n_out + 31) / 32);
   if (bid >= nt) {
-    const int i = (bid - nt) * 256 + threadIdx.x;
+    const int i = (bid - nt) * 256 + tid;
     if (i < a.n_out) a.b[i] = adam_value(q, a.b[i], a.gb[i], a.mb[i], a.vb[i]);
     return;
   }
-  const int k0 = (bid % tk) * 32, o0 = (bid / tk) * 32, x = threadIdx.x & 31, y = threadIdx.x >> 5;
+  const int k0 = (bid % tk) * 32, o0 = (bid / tk) * 32, x = tid & 31, y = tid >> 5;
 #pragma unroll
   for (int j = y; j < 32; j += 8) {
     const int o = o0 + j, k = k0 + x;
@@ -694,10 +696,10 @@ int mlp_gemm(int M, int N, int K, const __nv_bfloat16* A, int lda, const __nv_bf
   const long long tiles = (long long)cdiv(N, tn) * cdiv(M, TBM);
   const unsigned grid = (unsigned)std::min<long long>(tiles, g_sm_count[dev]);  // one persistent CTA per SM
   if (slim)
-    ICON_LAUNCH_SMEM("mlp_gemm_tc", grid, kTcThreads, tc_smem(kSlimN, kSlimStages), s,
+    ICON_CHAIN_SMEM("mlp_gemm_tc", grid, kTcThreads, tc_smem(kSlimN, kSlimStages), s,
                      (gemm_tc<kSlimN, kSlimStages>), ta, tb, M, N, K, ep);
   else
-    ICON_LAUNCH_SMEM("mlp_gemm_tc", grid, kTcThreads, tc_smem(kWideN, kWideStages), s,
+    ICON_CHAIN_SMEM("mlp_gemm_tc", grid, kTcThreads, tc_smem(kWideN, kWideStages), s,
                      (gemm_tc<kWideN, kWideStages>), ta, tb, M, N, K, ep);
   return ICON_OK;
 }
@@ -713,17 +715,17 @@ void mlp_layer_prep(int rows, int cols, const float* dz32, const __nv_bfloat16* 
                     cudaStream_t s) {
   const PrepArgs a{rows, dz32, dz16, ldz, cols, db, dzT, h, ldh, hcols, hT, ldt};
   const unsigned grid = cdiv(cols, 32) + (unsigned)(rows / kTr) * (cdiv(cols, kTr) + cdiv(hcols, kTr));
-  ICON_LAUNCH("mlp_layer_prep", grid, kPrepThreads, s, layer_prep, a);
+  ICON_CHAIN("mlp_layer_prep", grid, kPrepThreads, s, layer_prep, a);
 }
 
 void mlp_gelu_backward(int rows, int cols, const float* dh, int ldd, const float* z, int ldz, float* dz32,
                        __nv_bfloat16* dz16, int ldo, cudaStream_t s) {
-  ICON_LAUNCH("mlp_gelu_backward", cdiv(rows, kRowWarps), 32 * kRowWarps, s, gelu_backward, rows, cols, dh, ldd, z, ldz,
+  ICON_CHAIN("mlp_gelu_backward", cdiv(rows, kRowWarps), 32 * kRowWarps, s, gelu_backward, rows, cols, dh, ldd, z, ldz,
               dz32, dz16, ldo);
 }
 
 void mlp_to_bf16(int rows, int cols, const float* in, int ldi, __nv_bfloat16* out, int ldo, cudaStream_t s) {
-  ICON_LAUNCH("mlp_to_bf16", cdiv(rows, kRowWarps), 32 * kRowWarps, s, to_bf16, rows, cols, in, ldi, out, ldo);
+  ICON_CHAIN("mlp_to_bf16", cdiv(rows, kRowWarps), 32 * kRowWarps, s, to_bf16, rows, cols, in, ldi, out, ldo);
 }
 
 void mlp_adam(AdamLayers& ly, const AdamScal& q, cudaStream_t s) {
@@ -732,7 +734,7 @@ void mlp_adam(AdamLayers& ly, const AdamScal& q, cudaStream_t s) {
     n += (int)(cdiv(a.n_in, 32) * cdiv(a.n_out, 32) + cdiv(a.n_out, 256));
     a.block_end = n;
   }
-  ICON_LAUNCH("mlp_adam", (unsigned)n, 256, s, adam_update, ly, q);
+  ICON_CHAIN("mlp_adam", (unsigned)n, 256, s, adam_update, ly, q);
 }
 
 }  // namespace icon
@@ -745,7 +747,7 @@ namespace {
 __global__ void mse_kernel(int B, int n_out, const float* __restrict__ y, int ldy, const float* __restrict__ t,
                            int ldt, float* __restrict__ dy, __nv_bfloat16* __restrict__ dy16, int lddy,
                            double* __restrict__ rowloss) {
-  const int r = blockIdx.x * kRowWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int r = (int)after_previous(blockIdx.x * kRowWarps + (threadIdx.x >> 5)), lane = threadIdx.x & 31;
   if (r >= B) return;
   const float scale = 2.0f / ((float)B * (float)n_out);
   double s = 0.0;
@@ -768,7 +770,7 @@ __global__ void mse_kernel(int B, int n_out, const float* __restrict__ y, int ld
 
 void mlp_mse(int B, int n_out, const float* y, int ldy, const float* t, int ldt, float* dy, __nv_bfloat16* dy16,
              int lddy, double* rowloss, cudaStream_t s) {
-  ICON_LAUNCH("mlp_mse", (unsigned)((B + kRowWarps - 1) / kRowWarps), 32 * kRowWarps, s, mse_kernel, B, n_out, y, ldy,
+  ICON_CHAIN("mlp_mse", (unsigned)((B + kRowWarps - 1) / kRowWarps), 32 * kRowWarps, s, mse_kernel, B, n_out, y, ldy,
               t, ldt, dy, dy16, lddy, rowloss);
 }
 
