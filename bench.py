@@ -59,17 +59,17 @@ def hbm_peak():
         return HBM_FALLBACK_GBS, "fallback"
 
 
-# FP64 flops per unit (FMA = 2, add/mul = 1, a reciprocal = its FP64 add and
+# FP64 flops per unit (FMA = 2, add/mul = 1, a reciprocal or a square root =
 # two FMAs), counted from the arithmetic each kernel evaluates; the unit is
 # one (point, level).  va_cell_vert: the mean of its predictor and corrector
 # forms per unit of its combined cell and vertex launch.
 FLOPS_PER_UNIT = {
     "va_edge_pre": 15, "va_cell_vert": 14, "va_edge_tend": 21, "va_cell_w": 11,
-    "sn_cell_grad": 32, "sn_edge_pred": 24, "sn_cell_div": 5, "sn_cell_fluxdiv": 27,
+    "sn_cell_grad": 21, "sn_edge_pred": 24, "sn_cell_div": 5, "sn_cell_fluxdiv": 27,
     "sn_edge_flux": 6, "sn_cell_fluxsum": 12,
-    "sn_column_pred": 83, "sn_edge_corr": 11, "sn_column_corr": 84,
-    "diff_div_curl_uv": 30, "diff_edge_smag": 46, "diff_second": 30,
-    "diff_edge_update": 12, "diff_cell_update": 12, "va_concorr": 20,
+    "sn_column_pred": 81, "sn_edge_corr": 11, "sn_column_corr": 82,
+    "diff_div_curl_uv": 30, "diff_edge_smag": 40, "diff_second": 30,
+    "diff_edge_update": 11, "diff_cell_update": 18, "va_concorr": 20,
 }
 
 SUFFIXES = ("_f32", "_terrain", "_mx64", "_mx")
@@ -345,8 +345,9 @@ DRAM_PER_UNIT = {
     }}
 
 # The files whose code runs on the device in the timed steps.
-KERNEL_SOURCES = ("kernels_stencil.cu", "kernels_column.cu", "column_kernel.cuh", "kernels_column_terrain.cu",
-                  "kernels_diag.cu", "mlp.cu", "learned.cu", "dfloat.cuh", "kernels.h", "internal.h")
+KERNEL_SOURCES = ("kernels_stencil.cu", "stencil_quad.cuh", "kernels_column.cu", "column_kernel.cuh",
+                  "kernels_column_terrain.cu", "kernels_diag.cu", "mlp.cu", "learned.cu", "dfloat.cuh", "fp64.cuh",
+                  "kernels.h", "internal.h")
 
 
 def per_step_units(name, nc, ne, nlev):
@@ -406,10 +407,11 @@ def dram_measured(leg, prof, nsteps, ms_per_step, sizes, nlev, ndyn):
 
 # FP64 instructions per unit (DADD + DMUL + DFMA) where ncu counted them
 # (`smsp__sass_thread_inst_executed_op_{dadd,dmul,dfma}_pred_on`, R2B5 L90, the
-# sources of DRAM_PER_UNIT): the FP64 pipe issues one of any kind per slot, so
-# the instruction rate against the pipe's (half the FMA flop rate) is how busy
-# the pipe is, whatever the mix of adds and FMAs.
-FP64_INSTR_PER_UNIT = {"sn_column_pred": 59.1, "sn_column_corr": 60.0}
+# predictor in 8-level and the corrector in 4-level chunks): the FP64 pipe
+# issues one of any kind per slot, so the instruction rate against the pipe's
+# (half the FMA flop rate) is how busy the pipe is, whatever the mix of adds
+# and FMAs.
+FP64_INSTR_PER_UNIT = {"sn_column_pred": 56.9, "sn_column_corr": 63.5}
 
 # The column solve's predictor and corrector launches are one kernel (one
 # function, two forms); the roofline treats them together.

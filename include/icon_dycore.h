@@ -342,8 +342,8 @@ int icon_dycore_sizes(const icon_dycore_t* dycore, int32_t* nlev, int32_t* n_cel
  * whole step, which icon_dycore_create allocates, no longer fit.  Such a
  * caller can still run this solve on arrays it owns.
  *
- * It runs the same column kernel as icon_nh_solve (one thread per column,
- * Thomas elimination, Rayleigh damping, back-substitution, linearised
+ * It runs the same column kernel as icon_nh_solve (several threads per
+ * column, Thomas elimination, Rayleigh damping, back-substitution, linearised
  * equation of state) for n_cols independent columns of nlev levels:
  *   z_ifc [nlev+1] HOST, half-level heights as for icon_dycore_create; read
  *          during the call only (it is passed to the GPU by value);
