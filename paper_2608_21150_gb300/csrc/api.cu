@@ -294,7 +294,7 @@ bool grid_complete(const GridT<T>& g) {
                      g.upw_s, g.cpd_inv_d, g.hinv_d, g.d_o_l, g.lap_s, g.e2c_wd};
   for (const void* q : p)
     if (!q) return false;
-  if (std::is_same<T, double>::value && (!g.grad_nb || !g.grad_b || !g.smag_c)) return false;
+  if (std::is_same<T, double>::value && (!g.grad_nb || !g.grad_b || !g.grad_m || !g.smag_c)) return false;
   return true;
 }
 
@@ -597,13 +597,17 @@ int create_dycore(const icon_grid_t* grid, int nlev, const double* z_ifc, const 
     tenh64[e] = p->hdiff_tenh_fac * h.edge_area[e];
   }
   // cells by their place in the connectivity, as the kernel reads them
-  for (int c = 0; c < nc; ++c)
+  std::vector<unsigned char> grad_m(nc);
+  for (int c = 0; c < nc; ++c) {
+    grad_m[c] = (unsigned char)grad_nb[3 * (size_t)c + 2];
     for (int j = 0; j < 3; ++j) grad_nb[3 * (size_t)c + j] = h.c2e2c[3 * (size_t)c + grad_nb[3 * (size_t)c + j]];
+  }
   en.g64 = grid->dev;
   en.g64.hinv_d = A.upload(hinv_d);
   en.g64.d_o_l = A.upload(d_o_l);
   en.g64.grad_nb = A.upload(grad_nb);
   en.g64.grad_b = A.upload(grad_b);
+  en.g64.grad_m = A.upload(grad_m);
   en.g64.smag_c = A.upload(smag_c);
   en.g64.lap_s = A.upload(lap_s);
   en.g64.e2c_wd = A.upload(e2c_wd);
@@ -1460,26 +1464,11 @@ int icon_dycore_debug_field(icon_dycore_t* d, const char* name, void* dst, int64
   if (!src) return fail(ICON_ERR_ARG, std::string("icon_dycore_debug_field: unknown field ") + name);
   if (bytes < (int64_t)n) return fail(ICON_ERR_ARG, "icon_dycore_debug_field: destination too small");
   CUDA_TRY(cudaMemcpy2DAsync(dst, width, src, pitch, width, rows, cudaMemcpyDeviceToDevice, d->stream));
-  CUDA_TRY(cudaStreamSynchronize(d->stream));
   if (!mixed && std::strcmp(name, "grad4") == 0) {
-    // from the cells' own basis to the x and y of their frames
-    const size_t plane = nc * nlev;
-    std::vector<double> f(4 * plane);
-    CUDA_TRY(cudaMemcpy(f.data(), dst, n, cudaMemcpyDeviceToHost));
-    for (size_t c = 0; c < nc; ++c) {
-      int nb[3];
-      double b4[4];
-      const double* G = &h.grad_c[6 * c];
-      grad_basis(G, nb, b4);
-      for (size_t i = c * nlev; i < (c + 1) * nlev; ++i)
-        for (double* p = &f[i]; p <= &f[2 * plane + i]; p += 2 * plane) {
-          const double ga = p[0], gb = p[plane];
-          p[0] = G[2 * nb[0]] * ga + G[2 * nb[1]] * gb;
-          p[plane] = G[2 * nb[0] + 1] * ga + G[2 * nb[1] + 1] * gb;
-        }
-    }
-    CUDA_TRY(cudaMemcpy(dst, f.data(), n, cudaMemcpyHostToDevice));
+    launch_gradient_frame(d->en, static_cast<double*>(dst), d->stream);
+    CUDA_TRY(cudaGetLastError());
   }
+  CUDA_TRY(cudaStreamSynchronize(d->stream));
   return ICON_OK;
 }
 

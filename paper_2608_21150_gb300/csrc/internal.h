@@ -33,6 +33,7 @@ struct GridT {
   // vectors, grad = G_a A + G_b B, where G_m = alpha G_a + beta G_b
   const int* grad_nb;    // [nc*3] the neighbours a, b, m
   const double* grad_b;  // [nc*4] alpha, beta, 1 + alpha, 1 + beta
+  const unsigned char* grad_m;  // [nc] the place j of m; a and b are the next two, cyclically (read back only)
   const T* lap_s;   // [nc]   sum_j lap_c_j (the FP64 divergence Laplacian in the same form)
   const T* e2c_wd;  // [nc*3] e2c_w times 1/d of that edge (the sum of the edges' w advection)
   const T* k4w_c;   // [nc]   hdiff_w_k4 * A_c^2

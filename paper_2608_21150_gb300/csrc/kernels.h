@@ -182,6 +182,9 @@ void launch_substep(const Engine& en, const Ctx<T>& x, const StateView& st, cuda
 // Row A10: diffusion over dtime, state updated in place.
 template <class T>
 void launch_diffusion(const Engine& en, const Ctx<T>& x, const StateView& st, cudaStream_t s);
+// FP64 mode: four planes of gradient coefficients in the cells' own bases (f, a
+// copy of the work field) to the x and y of their frames, in place.
+void launch_gradient_frame(const Engine& en, double* f, cudaStream_t s);
 // Mixed mode: FP32 mirrors from the FP64 state.
 void launch_refresh_mirrors(const Engine& en, const StateView& st, cudaStream_t s);
 // Row A7: vertically implicit column solve (corrector = 0: the predicted state

@@ -674,6 +674,23 @@ __global__ void sn_cell_grad(GridT<double> g, VertT<double> v, const double* __r
   grad4[3 * n + i] = fma(G[1], tm, fma(-G[3], t, theta[ib]));
 }
 
+// The same planes read back: from (A, B) to the x and y of the cell's frame, in
+// place, each a sum of two rounded products.
+__global__ void gradient_frame(GridT<double> g, int nlev, double* __restrict__ f) {
+  int c, k;
+  if (!flat_index(g.nc, nlev, c, k)) return;
+  const size_t n = (size_t)g.nc * nlev;
+  const int m = g.grad_m[c], a = (m + 1) % 3, b = (m + 2) % 3;
+  const double* G = g.grad_c + 6 * (size_t)c;
+  double* p = f + (size_t)c * nlev + k;
+#pragma unroll
+  for (int j = 0; j < 2; ++j, p += 2 * n) {
+    const double ga = p[0], gb = p[n];
+    p[0] = __dadd_rn(__dmul_rn(G[2 * a], ga), __dmul_rn(G[2 * b], gb));
+    p[n] = __dadd_rn(__dmul_rn(G[2 * a + 1], ga), __dmul_rn(G[2 * b + 1], gb));
+  }
+}
+
 // -------------------------------------------------------------------------
 // A6 (predictor edges): upwind rho_e/theta_e from the back trajectory over
 // dt/2, horizontal pressure gradient with the extrapolated exner perturbation,
@@ -1365,6 +1382,11 @@ const char* const kStencilNames[kNumStencils] = {
     "va_edge_pre", "va_cell_vert", "va_edge_tend", "va_cell_w", "sn_cell_grad", "sn_edge_pred", "sn_cell_div",
     "sn_cell_fluxdiv", "sn_edge_corr", "diff_div_curl_uv", "diff_edge_smag", "diff_second", "diff_edge_update",
     "diff_cell_update", "va_concorr", "sn_edge_flux"};
+
+void launch_gradient_frame(const Engine& en, double* f, cudaStream_t s) {
+  const int nlev = en.v.nlev;
+  gradient_frame<<<blocks_for((long long)en.g64.nc * nlev, kThreads), kThreads, 0, s>>>(en.g64, nlev, f);
+}
 
 void launch_refresh_mirrors(const Engine& en, const StateView& st, cudaStream_t s) {
   const int nlev = en.v.nlev;
