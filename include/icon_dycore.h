@@ -128,8 +128,12 @@ typedef struct icon_dycore_params {
   int32_t autotune;        /* logical: pick per-kernel launch shapes at create time */
   int32_t synchronous;     /* logical: return only after the GPU work ended */
   void* stream;            /* cudaStream_t to enqueue on; NULL = default stream */
-  int32_t column_chunk;    /* levels per shared-memory chunk of the column solve: 4, 6 or 8;
-                              0 = 4, or the autotuner's choice when autotune is set */
+  int32_t column_chunk;    /* levels per shared-memory chunk of the column solve: 4, 6 or 8,
+                              in CTAs of 32 columns.  0: below 19 456 cells CTAs of 16
+                              columns in chunks of 8, the faster form there; from there on
+                              8 (predictor) and 4 (corrector), or the autotuner's choice
+                              for each when autotune is set.  The results are the same
+                              bits in every form */
   /* steep terrain (Sec. 4.1: the dycore runs over real orography; its diffusion
    * raises the coefficients for strong near-surface temperature gradients) */
   int32_t steep_hpg;       /* logical, terrain only: the horizontal pressure gradient at
@@ -305,10 +309,15 @@ int icon_dycore_debug_field(icon_dycore_t* dycore, const char* name, void* dst, 
 
 /* The launch shapes in use (picked by the autotuner when params.autotune is
  * set): writes a NUL-terminated text "name=threads,...;column_chunk=K" of at
- * most len bytes into buf (HOST).  The autotuner runs one step of every
- * kernel on a temporary uniform state at create time with each candidate
- * (128, 256, 512 threads per CTA for the stencils; 4, 6 or 8 levels per
- * shared-memory chunk for the column solve) and keeps the fastest per kernel. */
+ * most len bytes into buf (HOST).  The list ends in column_threads, the column
+ * solve's threads per CTA; K is its levels per shared-memory chunk.  Both are
+ * the predictor's; between the two stand ";column_columns=C" (columns per CTA),
+ * ";column_corrector_threads=T" and ";column_corrector_chunk=K".  The
+ * autotuner runs one step of every kernel on a temporary uniform state at
+ * create time with each candidate (128, 256, 512 threads per CTA for the
+ * stencils; 4, 6 or 8 levels per chunk for the predictor and the corrector of
+ * the column solve, where its form for small grids does not fix them) and keeps
+ * the fastest per kernel. */
 int icon_dycore_launch_config(const icon_dycore_t* dycore, char* buf, int32_t len);
 
 /* Block until all work enqueued by this dycore has finished. */

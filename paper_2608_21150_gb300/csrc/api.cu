@@ -913,6 +913,7 @@ int create_dycore(const icon_grid_t* grid, int nlev, const double* z_ifc, const 
   }
   for (int k = 0; k < kNumStencils; ++k) en.threads[k] = 256;
   en.col_narrow = p->column_chunk == 0 && narrow_columns(nc);
+  if (en.col_narrow) en.col_kc[0] = en.col_kc[1] = 8;  // its only form
   if (p->autotune) {
     int rc = autotune(d);
     if (rc != ICON_OK) {
@@ -1518,13 +1519,12 @@ int icon_dycore_launch_config(const icon_dycore_t* d, char* buf, int32_t len) {
     if (d->en.shape[k] >= 0) s += d->en.shape[k] ? "w" : "t";
     s += ",";
   }
-  s += "column_columns=" + std::to_string(d->en.col_narrow ? kColNarrow : kColWide) + ";column_chunk=";
-  if (d->en.col_narrow)
-    s += "8";
-  else if (d->en.col_kc[0] == d->en.col_kc[1])
-    s += std::to_string(d->en.col_kc[0]);
-  else
-    s += std::to_string(d->en.col_kc[0]) + "/" + std::to_string(d->en.col_kc[1]);
+  const Engine& en = d->en;
+  s += "column_threads=" + std::to_string(column_threads(en, 0));
+  s += ";column_columns=" + std::to_string(en.col_narrow ? kColNarrow : kColWide);
+  s += ";column_corrector_threads=" + std::to_string(column_threads(en, 1));
+  s += ";column_corrector_chunk=" + std::to_string(en.col_kc[1]);
+  s += ";column_chunk=" + std::to_string(en.col_kc[0]);
   std::snprintf(buf, (size_t)len, "%s", s.c_str());
   return ICON_OK;
 }

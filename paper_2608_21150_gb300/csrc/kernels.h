@@ -193,6 +193,8 @@ void launch_refresh_mirrors(const Engine& en, const StateView& st, cudaStream_t 
 template <class T>
 void launch_column(const Engine& en, int corrector, const StateView& st, const T* ddt_w0, const T* ddt_w1,
                    cudaStream_t s);
+// Threads per CTA of the form that launch takes.
+int column_threads(const Engine& en, int corrector);
 // The same over terrain: per-column metrics (en.v.colt) and the solve in
 // w - wcc, wcc the contravariant correction (cells, half levels, type T).
 template <class T>

@@ -32,6 +32,14 @@ void launch_column(const Engine& en, int corrector, const StateView& st, const T
     launch_col_form<T, ColArith<T>, false>(en, corrector, a, name, s);
 }
 
+int column_threads(const Engine& en, int corrector) {
+  int n = 0;
+  with_col_form(en.col_kc[corrector ? 1 : 0], en.col_narrow, [&](auto kc, auto cw, auto rl) {
+    n = ColForm<double, decltype(kc)::value, decltype(cw)::value, decltype(rl)::value, true, false>::NT;
+  });
+  return n;
+}
+
 template void launch_column<double>(const Engine&, int, const StateView&, const double*, const double*, cudaStream_t);
 template void launch_column<float>(const Engine&, int, const StateView&, const float*, const float*, cudaStream_t);
 
