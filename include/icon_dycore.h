@@ -131,7 +131,7 @@ typedef struct icon_dycore_params {
   int32_t column_chunk;    /* levels per shared-memory chunk of the column solve: 4, 6 or 8,
                               in CTAs of 32 columns.  0: below 19 456 cells CTAs of 16
                               columns in chunks of 8, the faster form there; from there on
-                              8 (predictor) and 4 (corrector), or the autotuner's choice
+                              8 (4 at up to four levels; predictor) and 4 (corrector), or the autotuner's choice
                               for each when autotune is set.  The results are the same
                               bits in every form */
   /* steep terrain (Sec. 4.1: the dycore runs over real orography; its diffusion

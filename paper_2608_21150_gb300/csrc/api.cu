@@ -913,7 +913,10 @@ int create_dycore(const icon_grid_t* grid, int nlev, const double* z_ifc, const 
   }
   for (int k = 0; k < kNumStencils; ++k) en.threads[k] = 256;
   en.col_narrow = p->column_chunk == 0 && narrow_columns(nc);
-  if (en.col_narrow) en.col_kc[0] = en.col_kc[1] = 8;  // its only form
+  if (en.col_narrow)
+    en.col_kc[0] = en.col_kc[1] = 8;  // its only form
+  else if (nlev <= 4)
+    en.col_kc[0] = 4;  // chunks of 8 mostly empty: 2.9 instead of 2.8 ms a step at R2B6 and two levels, FP64
   if (p->autotune) {
     int rc = autotune(d);
     if (rc != ICON_OK) {

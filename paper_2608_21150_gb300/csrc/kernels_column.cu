@@ -2,6 +2,7 @@
 // column_kernel.cuh) and the allocation-free entry point.
 #include <cuda_runtime.h>
 
+#include <climits>
 #include <cmath>
 #include <mutex>
 #include <string>
@@ -185,8 +186,22 @@ constexpr int kNoallocMaxDevices = 64;
 std::mutex g_noalloc_mutex;
 double* g_noalloc_ptr[kNoallocMaxDevices] = {};
 
-using NoallocWide = ColForm<double, 8, kColWide, 2, true, false>;
-using NoallocNarrow = ColForm<double, 8, kColNarrow, 1, true, false>;
+// Runs f on the form of the solve for these sizes (chunk, columns per CTA, levels
+// a worker).  At up to four levels the wide form's chunks of 8 stage tiles that
+// are mostly empty and leave their workers without a level: 349 000 columns of 2
+// levels to 209 000 of 4 took 114-173 us in them, 102-159 with one thread
+// walking each column, 75-132 in chunks of 2 (both arithmetics, both forms).
+constexpr int kFewLevels = 4;
+template <class Fn>
+void with_noalloc_form(int n_cols, int nlev, Fn&& f) {
+  using std::integral_constant;
+  if (narrow_columns(n_cols))
+    f(integral_constant<int, 8>{}, integral_constant<int, kColNarrow>{}, integral_constant<int, 1>{});
+  else if (nlev <= kFewLevels)
+    f(integral_constant<int, 2>{}, integral_constant<int, kColWide>{}, integral_constant<int, 1>{});
+  else
+    f(integral_constant<int, 8>{}, integral_constant<int, kColWide>{}, integral_constant<int, 2>{});
+}
 
 // Once per device, with that device current: the device address of the
 // static array (its host-side name is only a stand-in) and the kernel's
@@ -206,10 +221,14 @@ int noalloc_setup(double** out) {
     auto set = [&](auto kernel, size_t bytes) {
       if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     };
-    set(sn_column<double, double, 8, kColWide, 2, -1, false, true>, NoallocWide::bytes);
-    set(sn_column<double, dws, 8, kColWide, 2, -1, false, true>, NoallocWide::bytes);
-    set(sn_column<double, double, 8, kColNarrow, 1, -1, false, true>, NoallocNarrow::bytes);
-    set(sn_column<double, dws, 8, kColNarrow, 1, -1, false, true>, NoallocNarrow::bytes);
+    for (int n : {1, INT_MAX})
+      for (int nlev : {2, kFewLevels + 1})
+        with_noalloc_form(n, nlev, [&](auto kc, auto cw, auto rl) {
+          constexpr int KC = decltype(kc)::value, CW = decltype(cw)::value, RL = decltype(rl)::value;
+          using F = ColForm<double, KC, CW, RL, true, false>;
+          set(sn_column<double, double, KC, CW, RL, -1, false, true>, F::bytes);
+          set(sn_column<double, dws, KC, CW, RL, -1, false, true>, F::bytes);
+        });
     if (e != cudaSuccess)
       return report_error(ICON_ERR_CUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));
     g_noalloc_ptr[dev] = ptr;
@@ -331,21 +350,17 @@ extern "C" int icon_column_solve_noalloc(int32_t n_cols, int32_t nlev, const dou
   a.theta_o = theta_new;
   const bool dw = p->precision == ICON_PREC_MIXED;  // the mixed mode's double-word FP32 arithmetic
   const int corrector = corr ? 1 : 0;
-  if (narrow_columns(n_cols)) {
-    using F = NoallocNarrow;
-    const unsigned blocks = (unsigned)((n_cols + kColNarrow - 1) / kColNarrow);
+  with_noalloc_form(n_cols, nlev, [&](auto kc, auto cw, auto rl) {
+    constexpr int KC = decltype(kc)::value, CW = decltype(cw)::value, RL = decltype(rl)::value;
+    using F = ColForm<double, KC, CW, RL, true, false>;
+    const unsigned blocks = (unsigned)((n_cols + CW - 1) / CW);
     if (dw)
-      launch_chained(blocks, F::NT, F::bytes, stream, sn_column<double, dws, 8, kColNarrow, 1, -1, false, true>, n_cols, v, s, corrector, a);
+      launch_chained(blocks, F::NT, F::bytes, stream, sn_column<double, dws, KC, CW, RL, -1, false, true>, n_cols, v, s,
+                     corrector, a);
     else
-      launch_chained(blocks, F::NT, F::bytes, stream, sn_column<double, double, 8, kColNarrow, 1, -1, false, true>, n_cols, v, s, corrector, a);
-  } else {
-    using F = NoallocWide;
-    const unsigned blocks = (unsigned)((n_cols + kColWide - 1) / kColWide);
-    if (dw)
-      launch_chained(blocks, F::NT, F::bytes, stream, sn_column<double, dws, 8, kColWide, 2, -1, false, true>, n_cols, v, s, corrector, a);
-    else
-      launch_chained(blocks, F::NT, F::bytes, stream, sn_column<double, double, 8, kColWide, 2, -1, false, true>, n_cols, v, s, corrector, a);
-  }
+      launch_chained(blocks, F::NT, F::bytes, stream, sn_column<double, double, KC, CW, RL, -1, false, true>, n_cols, v,
+                     s, corrector, a);
+  });
   e = cudaGetLastError();
   if (e != cudaSuccess) return report_error(ICON_ERR_CUDA, std::string(fn) + cudaGetErrorString(e));
   if (p->synchronous) {
