@@ -240,6 +240,20 @@ struct WorkT {
   T* w_v;                  // half levels
 };
 
+// Columns per CTA of the column solve: 32 (a warp's lanes are 32 columns, the
+// elimination runs at full width) once they give every SM four CTAs; below
+// that 16, so that a small grid spreads over more SMs.  Measured, predictor,
+// wide (chunks of 8) against narrow: FP64 R2B2 L30 35 / 27 us, R2B3 L31 49 /
+// 43, R2B4 L65 206 / 214; mixed R2B3 L31 30 / 26, R2B4 L65 103 / 127.
+constexpr int kColWide = 32, kColNarrow = 16;
+constexpr int kWideFrom = 4 * 152 * kColWide;  // columns from which the wide form is used
+constexpr bool narrow_columns(int nc) { return nc < kWideFrom; }
+// Column-levels that the solve's scratch holds per plane: whole groups of columns.
+constexpr size_t scratch_points(int nc, int nlev) {
+  const size_t group = narrow_columns(nc) ? kColNarrow : kColWide;
+  return (nc + group - 1) / group * group * nlev;
+}
+
 // FP64 work of the column solve and the predicted state.
 struct DevWork {
   double *div_m, *div_t;                  // cells: flux divergences (FP64 sums; double-word pairs in mixed mode)

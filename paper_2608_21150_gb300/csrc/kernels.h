@@ -118,14 +118,6 @@ struct Ctx {
 // The fused velocity-advection kernel's shared-memory limit for these patches.
 cudaError_t init_va_fused(const VaPatchT& pt);
 
-// Columns per CTA of the column solve: 32 (a warp's lanes are 32 columns, the
-// elimination runs at full width) once they give every SM four CTAs; below
-// that 16, so that a small grid spreads over more SMs.  Measured, predictor,
-// wide (chunks of 8) against narrow: FP64 R2B2 L30 35 / 27 us, R2B3 L31 49 /
-// 43, R2B4 L65 206 / 214; mixed R2B3 L31 30 / 26, R2B4 L65 103 / 127.
-constexpr int kColWide = 32, kColNarrow = 16;
-inline bool narrow_columns(int nc) { return nc < 4 * 152 * kColWide; }
-
 // Device-side state of one dycore: FP64 factors and column-solve work, the
 // FP32 mirrors (mixed mode) and the stencil context of the active mode.
 // The mixed modes (FP32 stencils) differ only in the column solve's arithmetic.

@@ -72,11 +72,13 @@ constexpr size_t kNoallocPlanes = 8;                   // kScratchPlanes
 constexpr size_t kNoallocMaxPoints = (kNoallocDoubles - kNoallocCoef) / kNoallocPlanes;
 static_assert(kNoallocMaxPoints == 1047232, "the limit stated in icon_dycore.h");
 static_assert(kNoallocPlanes == kScratchPlanes, "planes of the column solve's scratch");
-// The scratch holds whole groups of columns on nlev levels: at most (n_cols +
-// 15) nlev column-levels in the narrow form, which 15 nlev <= n_cols keeps
-// within n_cols (nlev + 1) (fewer columns than that stay below the limit), and (n_cols + 31) nlev in the wide one (n_cols >= 19 456, so nlev <= 52).
+// The scratch holds whole groups of columns on nlev levels.  Narrow form: at most
+// (n_cols + 15) nlev column-levels, within n_cols (nlev + 1) once 15 nlev <=
+// n_cols, and fewer columns than that stay below the limit.  Wide form:
+// (n_cols + 31) nlev with n_cols >= kWideFrom, so nlev <= limit / kWideFrom and
+// 31 nlev <= n_cols.  The call checks the sum itself too (scratch_points).
 static_assert(kColNarrow == 16 && 15 * (size_t)kNoallocMaxLev * (kNoallocMaxLev + 1) < kNoallocMaxPoints &&
-                  31 * (kNoallocMaxPoints / (4 * 152 * kColWide)) <= 4 * 152 * kColWide,
+                  kColWide == 32 && 31 * (kNoallocMaxPoints / kWideFrom) <= kWideFrom,
               "the groups' spare columns fit");
 static_assert(8 * kNoallocStride + 8 * (kNoallocMaxLev + 1) <= kNoallocLevHL, "column coefficients fit");
 static_assert(kNoallocLevHL + 16 * (kNoallocMaxLev + 1) <= kNoallocCoef, "level table fits");
@@ -261,6 +263,8 @@ extern "C" int icon_column_solve_noalloc(int32_t n_cols, int32_t nlev, const dou
     return report_error(ICON_ERR_ARG, std::string(fn) + "n_cols*(nlev+1) = " + std::to_string(points) +
                                           " exceeds the static scratch of " + std::to_string(kNoallocMaxPoints) +
                                           " column-levels (64 MiB)");
+  if (scratch_points(n_cols, nlev) > kNoallocMaxPoints)
+    return report_error(ICON_ERR_ARG, std::string(fn) + "the groups of columns exceed the static scratch");
   for (int k = 0; k <= nlev; ++k)
     if (!std::isfinite(z_ifc[k])) return report_error(ICON_ERR_ARG, std::string(fn) + "z_ifc not finite");
   for (int k = 0; k < nlev; ++k)
