@@ -661,6 +661,58 @@ def mixed_summary(m, f64, world, nsteps, area, sizes, nlev, ndyn, leg):
             "autotuned_launch_config": m["launch_config"]}
 
 
+# What the printed line keeps of the full record: readers that keep only the end
+# of a program's output get all of it (tests/test_bench_line_cpu.py).  The rest is
+# in the file that --details names.
+LINE_LIMIT = 2400  # characters
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+             "vs_baseline", "dtype", "data", "config", "gpu_launches", "clocks", "finite")
+LEG_KEYS = ("value", "speedup_vs_fp64", "finite", "rms_ps_pa", "rms_ps_pa_vs_fp64", "fallbacks_timed")
+
+
+def rounded(x, digits=5):
+    """x with its floats at `digits` significant digits, in dicts and lists too."""
+    if isinstance(x, float):
+        return float("%.*g" % (digits, x))
+    if isinstance(x, dict):
+        return {k: rounded(v, digits) for k, v in x.items()}
+    if isinstance(x, (list, tuple)):
+        return [rounded(v, digits) for v in x]
+    return x
+
+
+def picked(d, keys):
+    return {k: d[k] for k in keys if d.get(k) is not None} if d else None
+
+
+def result_line(full):
+    """The one line printed: the headline as measured, and of each leg its rate,
+    its error against FP64 and its measured share of the HBM bandwidth."""
+    def leg(m):
+        out = picked(m, LEG_KEYS)
+        if m and m.get("hbm_measured"):
+            out["hbm_frac"] = m["hbm_measured"]["frac"]
+        return out
+
+    line = {k: full[k] for k in LINE_KEYS}
+    line["e2e"] = picked(full["e2e"], ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "mean_value",
+                                       "median_value"))
+    more = {"hbm": picked(full["hbm"], ("achieved_gbs", "peak_gbs", "frac")),
+            "hbm_measured": picked(full["hbm_measured"], ("bytes_per_step", "achieved_gbs", "peak_gbs", "frac")),
+            "roofline": picked(full["roofline"], ("bound", "kernel", "achieved", "peak", "unit", "frac", "traffic"))}
+    if full["roofline"] and full["roofline"].get("fp64_issue"):
+        more["roofline"]["fp64_issue_frac"] = full["roofline"]["fp64_issue"]["frac"]
+    for k in ("mixed", "mixed_f64col", "mixed_learned"):
+        more[k] = leg(full[k])
+    mountain = full["mountain_r2b7"]
+    more["mountain_r2b7"] = {k: leg(mountain[k]) for k in ("fp64", "mixed", "mixed_learned")} if mountain else None
+    more["cpu_baseline"] = picked(full.get("cpu_baseline"), ("value", "unit", "cores", "kind", "extrapolated"))
+    if more["cpu_baseline"]:
+        more["cpu_baseline"]["sample"] = "one R2B4 L90 substep and diffusion, x16 (cells) and x5 (substeps)"
+    line.update(rounded({k: v for k, v in more.items() if v}))
+    return line
+
+
 def mountain_legs(P, args, dev, world):
     """The R2B7 L90 Gaussian-mountain configuration (dt 180 s): FP64, mixed and
     mixed + learned over terrain-following heights, timed steps each, the
@@ -835,7 +887,10 @@ def run_ours(args):
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
         line["cpu_baseline"] = cpu_baseline(nlev)
     if rank == 0:
-        print(json.dumps(line))
+        if args.details:
+            with open(args.details, "w") as fh:
+                json.dump(line, fh, indent=1)
+        print(json.dumps(result_line(line)))
     if world > 1:
         dist.destroy_process_group()
     return 0
@@ -847,6 +902,8 @@ def main():
     ap.add_argument("--steps", type=int, default=20)
     ap.add_argument("--warmup", type=int, default=3)
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
+    ap.add_argument("--details", help="write the full record (every kernel's times, launch shapes, training, notes) "
+                                      "to this file")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--legs", default="fp64,mixed,mixed_f64col,learned",
                     help="comma-separated legs to run (fp64, mixed, mixed_f64col, learned); the headline value is "
