@@ -661,6 +661,16 @@ def mixed_summary(m, f64, world, nsteps, area, sizes, nlev, ndyn, leg):
             "autotuned_launch_config": m["launch_config"]}
 
 
+def end_to_end(times, nbytes):
+    """The end-to-end record of host-array steps that took `times` seconds each:
+    the rate over all of them, and at their median."""
+    return {"value": len(times) / sum(times), "unit": "steps/s", "h2d_bytes_per_step": nbytes,
+            "d2h_bytes_per_step": nbytes, "median_value": 1.0 / statistics.median(times),
+            "step_ms": [round(1e3 * x, 2) for x in times],
+            "note": "value over the wall time of %d synchronous host-array steps (pinned host arrays, copies in and "
+                    "out inside each step); median_value at the median step" % len(times)}
+
+
 # What the printed line keeps of the full record: readers that keep only the end
 # of a program's output get all of it (tests/test_bench_line_cpu.py).  The rest is
 # in the file that --details names.
@@ -695,7 +705,7 @@ def result_line(full):
         return out
 
     line = {k: full[k] for k in LINE_KEYS}
-    line["e2e"] = picked(full["e2e"], ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "mean_value",
+    line["e2e"] = picked(full["e2e"], ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step",
                                        "median_value"))
     more = {"hbm": picked(full["hbm"], ("achieved_gbs", "peak_gbs", "frac")),
             "hbm_measured": picked(full["hbm_measured"], ("bytes_per_step", "achieved_gbs", "peak_gbs", "frac")),
@@ -843,11 +853,7 @@ def run_ours(args):
         finally:
             gc.enable()
         D2.close()
-        med = statistics.median(times)
-        e2e = {"value": 1.0 / med, "unit": "steps/s", "h2d_bytes_per_step": sb, "d2h_bytes_per_step": sb,
-               "mean_value": len(times) / sum(times), "step_ms": [round(1e3 * x, 2) for x in times],
-               "note": "value at the median wall time of %d synchronous host-array steps (pinned host arrays, "
-                       "copies in and out inside each step); mean_value over all of them" % len(times)}
+        e2e = end_to_end(times, sb)
     G.close()
     torch.cuda.empty_cache()
 

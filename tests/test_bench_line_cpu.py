@@ -28,8 +28,7 @@ def _full(B):
         "hbm_measured": hbm, "roofline": B.roofline(prof, nc, ne, nv, 90), "kernels": B.kernel_table(prof, 2),
         "autotuned_launch_config": "a" * 600, "steps_compared": 240, "mixed": leg, "mixed_f64col": leg,
         "mixed_learned": learned, "mountain_r2b7": {"config": {}, "fp64": leg, "mixed": leg, "mixed_learned": learned},
-        "e2e": {"value": x / 99, "unit": "steps/s", "h2d_bytes_per_step": 1536163840, "d2h_bytes_per_step": 1536163840,
-                "mean_value": x / 98, "median_value": x / 97, "step_ms": [x] * 10, "note": "n" * 200},
+        "e2e": B.end_to_end([x / 1000] * 9 + [x / 500], 1536163840),
         "gpu_launches": 123456, "clocks": clocks, "finite": True,
         "cpu_baseline": {"value": x, "unit": "steps/s", "cores": 16, "kind": "oracle", "sample": "s" * 400,
                          "extrapolated": True, "single_thread": {"value": x}}}
@@ -65,3 +64,13 @@ def test_the_line_of_a_run_without_legs():
     full.pop("cpu_baseline")
     line = json.loads(json.dumps(B.result_line(full)))
     assert line["value"] is None and line["e2e"] is None and "mixed" not in line
+
+
+def test_the_end_to_end_rate_counts_every_step():
+    if ROOT not in sys.path:
+        sys.path.insert(0, ROOT)
+    B = importlib.import_module("bench")
+    e = B.end_to_end([0.1] * 8 + [0.165, 0.164], 7)
+    assert abs(e["value"] - 10 / (0.8 + 0.165 + 0.164)) < 1e-12
+    assert abs(e["median_value"] - 10.0) < 1e-12
+    assert e["h2d_bytes_per_step"] == e["d2h_bytes_per_step"] == 7 and e["step_ms"][-2:] == [165.0, 164.0]
