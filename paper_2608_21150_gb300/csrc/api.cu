@@ -291,10 +291,10 @@ bool grid_complete(const GridT<T>& g) {
   const void* p[] = {g.c2e, g.c2e2c, g.e2c, g.e2v, g.e2c2v, g.e2c2e, g.v2e, g.v2c, g.div_c, g.lap_c, g.e2c_w,
                      g.grad_c, g.k4w_c, g.inv_d, g.inv_l, g.f_e, g.vt_w, g.upw, g.nt, g.inv_dn, g.smag_a, g.k4_a,
                      g.fdiv_e, g.ddamp_e, g.curl_v, g.c2v_w, g.uv_w, g.cell_area, g.uv_c, g.div_c_hl,
-                     g.upw_s, g.cpd_inv_d, g.hinv_d, g.d_o_l, g.lap_s, g.e2c_wd};
+                     g.upw_s, g.cpd_inv_d, g.hinv_d, g.d_o_l, g.e2c_wd};
   for (const void* q : p)
     if (!q) return false;
-  if (std::is_same<T, double>::value && (!g.grad_nb || !g.grad_b || !g.grad_m || !g.smag_c)) return false;
+  if (std::is_same<T, double>::value && (!g.lap_s || !g.grad_nb || !g.grad_b || !g.grad_m || !g.smag_c)) return false;
   return true;
 }
 
@@ -658,7 +658,6 @@ int create_dycore(const icon_grid_t* grid, int nlev, const double* z_ifc, const 
     g.inv_l = up(h.inv_l);
     g.hinv_d = up(hinv_d);
     g.d_o_l = up(d_o_l);
-    g.lap_s = up(lap_s);
     g.e2c_wd = up(e2c_wd);
     g.f_e = up(fe);
     g.vt_w = up(h.vt_w);

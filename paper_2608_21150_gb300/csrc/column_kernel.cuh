@@ -167,7 +167,6 @@ struct ColArgs {
   double *col, *w_o, *rho_o, *exner_o, *theta_o;
   // mixed mode: FP32 mirrors of the outputs (w; rho, theta_v perturbations)
   float *m_w, *m_rho, *m_th;
-  const double* rho_ref;
   // terrain: contravariant correction of the winds (cells, half levels)
   const T* wcc;
   // row stride of the fields of type T and of the mirrors
@@ -820,7 +819,6 @@ ColArgs<T> col_args(const Engine& en, int corrector, const StateView& st, const 
   a.div_m = wk.div_m;
   a.div_t = wk.div_t;
   a.col = wk.col;
-  a.rho_ref = en.rho_ref64;
   a.ldt = std::is_same<T, float>::value ? en.c32.v.ldh : en.c64.v.ldh;
   constexpr bool mixed = std::is_same<T, float>::value;
   if (corrector) {

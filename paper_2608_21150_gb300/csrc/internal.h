@@ -34,7 +34,7 @@ struct GridT {
   const int* grad_nb;    // [nc*3] the neighbours a, b, m
   const double* grad_b;  // [nc*4] alpha, beta, 1 + alpha, 1 + beta
   const unsigned char* grad_m;  // [nc] the place j of m; a and b are the next two, cyclically (read back only)
-  const T* lap_s;   // [nc]   sum_j lap_c_j (the FP64 divergence Laplacian in the same form)
+  const double* lap_s;  // [nc] FP64: sum_j lap_c_j (the divergence Laplacian as a weighted sum)
   const T* e2c_wd;  // [nc*3] e2c_w times 1/d of that edge (the sum of the edges' w advection)
   const T* k4w_c;   // [nc]   hdiff_w_k4 * A_c^2
   // edge coefficients
