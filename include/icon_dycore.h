@@ -149,7 +149,7 @@ typedef struct icon_dycore_params {
                                ground: the velocity tendencies (rows A1-A4) in one
                                kernel over patches of 128 cells, intermediates in
                                shared memory; the same bits as the four separate
-                               kernels, and on GB300 about 1.3x their time */
+                               kernels, and on GB300 about 2.2x their time */
 } icon_dycore_params_t;
 
 /* Writes the defaults (Sec. 4.1 names the scheme's parts, not its values;
@@ -378,7 +378,7 @@ int icon_dycore_sizes(const icon_dycore_t* dycore, int32_t* nlev, int32_t* n_cel
  * nlev <= 256 and n_cols*(nlev+1) <= 1 047 232 column-levels (at nlev = 90:
  * 11 508 columns); larger calls return ICON_ERR_ARG before any GPU work.
  * No cudaMalloc, cudaFree or other allocating call is made.  The vertical
- * metrics are computed on the device, by a one-thread kernel on the same
+ * metrics are computed on the device, by a kernel of one CTA on the same
  * stream, from z_ifc and the scalars passed by value.  The first call on
  * each device looks up the array's device address (cudaGetSymbolAddress)
  * and sets the kernel's shared-memory limit.  All calls share the array and

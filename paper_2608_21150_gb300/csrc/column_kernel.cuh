@@ -1,5 +1,6 @@
-// Row A7: vertically implicit solve of w, rho, exner and theta_v, one thread
-// per column (the tridiagonal Thomas sweep is sequential in the vertical).
+// Row A7: vertically implicit solve of w, rho, exner and theta_v, several
+// threads per column; only the tridiagonal Thomas sweep, which is sequential in
+// the vertical, has one.
 //
 // Equations (an ICON-type reading; the paper names the solver but gives no
 // formula, Sec. 4.1), for full levels k (dz) and interior half levels k (dzh),
@@ -22,13 +23,14 @@
 //   theta' = theta (rho/rho')(1 + (cvd/rd)(pr' - pr)/exner)
 //          = (dt rd/(cvd dz)) (exner - (cvd/rd) pr + (cvd/rd) pr') / (zb rho').
 //
-// Memory: the state is level-contiguous, so a thread walking its own column
+// Memory: the state is level-contiguous, so a warp whose lanes are columns
 // would read every 32-byte sector for 8 useful bytes.  Instead each CTA stages
-// chunks of KC levels (4, 6 or 8, picked by the autotuner for each form) of
-// every input through shared memory with coalesced asynchronous copies (a
-// column's chunk is a contiguous run), and stages its outputs the same way.
-// Each chunk's slice of the per-level table is staged with them (FP64 or
-// double-word): every thread of a warp reads the same level at the same time.
+// chunks of KC levels (4, 6 or 8, picked by the autotuner for the predictor and
+// the corrector) of every input through shared memory with coalesced
+// asynchronous copies (a column's chunk is a contiguous run), and stages its
+// outputs the same way.  Each chunk's slice of the per-level table is staged
+// with them (FP64 or double-word): a warp reads one level of it at a time, with
+// 16 columns per CTA two.
 // The scratch between the sweeps is laid out so that a thread reaches a
 // level's planes from one address and a warp's accesses are coalesced; it is
 // written as streaming data and read back evict-first, while the input rows
@@ -40,8 +42,9 @@
 // 27 / 27 us, R2B4 L65 FP64 277 / 287 -> 197 / 213 us, R2B6 L90 double-word
 // 1.87 / 2.64 -> 1.59 / 2.06 ms, R2B5 L90 double-word over terrain 1.09 / 1.36
 // -> 0.70 / 0.94 ms.  R2B6 L90 FP64 3.41 / 3.67 -> 3.31 / 3.58 ms: there both
-// keep the FP64 unit busy (a warp's FP64 instruction takes 19 cycles of the
-// SM; 57 to 61 of them a level), and only the reciprocal's operations counted.
+// keep the FP64 unit busy (a warp's FP64 instruction takes 16 cycles of the SM
+// at best and 19 here; 56.9 of them a level in the predictor's chunks of 8, 63.5
+// in the corrector's of 4), and only the reciprocal's operations counted.
 //
 // This header holds the kernel template and its helpers; kernels_column.cu
 // instantiates the flat-ground forms (and the allocation-free entry point),

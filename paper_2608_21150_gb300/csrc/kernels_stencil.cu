@@ -694,11 +694,10 @@ __global__ void gradient_frame(GridT<double> g, int nlev, double* __restrict__ f
 // -------------------------------------------------------------------------
 // A6 (predictor edges): upwind rho_e/theta_e from the back trajectory over
 // dt/2, horizontal pressure gradient with the extrapolated exner perturbation,
-// and the vn predictor.  FP64 mode reads totals; mixed mode reads the
-// perturbations of rho and theta_v and adds the reference back.  The
-// extrapolated exner perturbations come per cell from sn_cell_grad; their
-// difference across the edge is taken in FP64 (double-word FP32 in mixed
-// mode): neighbouring perturbations agree to 4-5 digits, more than FP32 carries.
+// and the vn predictor, FP64 (the mixed modes: sn_edge_pred_q in
+// stencil_quad.cuh).  The extrapolated exner perturbations come per cell from
+// sn_cell_grad; their difference across the edge is taken in FP64, since
+// neighbouring perturbations agree to 4-5 digits.
 // -------------------------------------------------------------------------
 // Over terrain (kTerr) the pressure gradient is taken along the true
 // horizontal: the along-level difference minus the slope of the full level

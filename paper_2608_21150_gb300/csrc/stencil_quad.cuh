@@ -363,8 +363,11 @@ __global__ void sn_cell_grad_q(GridT<float> g, VertT<float> v, const float* __re
   st4(grad4 + 3 * n + i, o);
 }
 
-// A6, as sn_edge_pred.  A quad's levels mostly share their upwind cell: its
-// fields come as quads then, else level by level.
+// A6, as sn_edge_pred, from the perturbations of rho and theta_v, with the
+// reference added back; the difference of the exner perturbations across the
+// edge is taken of double-word pairs (neighbours agree to 4-5 digits, more than
+// FP32 carries).  A quad's levels mostly share their upwind cell: its fields come
+// as quads then, else level by level.
 template <bool kTerr>
 __global__ void sn_edge_pred_q(GridT<float> g, VertT<float> v, ScalT<float> sc, const float* __restrict__ vn,
                                const float* __restrict__ vt, const float* __restrict__ ddt_vn,
@@ -513,8 +516,8 @@ __global__ void sn_cell_div_q(GridT<float> g, VertT<float> v, const float* __res
 //   vf_e = vn_e + divflux (D_c1 - D_c0)/d_e,  F_e = rho_e vf_e,
 //   div_m = sum s l F / A,  div_t = sum s l F theta_e / A
 // Over terrain (kTerr) each flux carries its edge layer thickness over the
-// cell's, fx_ratio = dz_e / dz_c.  pairs: an even nlev, so that two levels'
-// results are one aligned store.
+// cell's, fx_ratio = dz_e / dz_c.  With an even nlev two levels' results are one
+// aligned store.
 template <bool kTerr>
 __global__ void sn_cell_fluxdiv_q(GridT<float> g, VertT<float> v, const float* __restrict__ vn,
                                   const float* __restrict__ divd, const float* __restrict__ rho_e,
