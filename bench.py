@@ -309,39 +309,39 @@ def config_dict(prec):
 
 
 # ---------------------------------------------------------------------------
-# DRAM traffic per unit of every kernel, from one-kernel ncu captures
-# (dram__bytes_read.sum + dram__bytes_write.sum of one launch, -c 1; the
-# column solve's predictor and corrector -c 2) at R2B5 L90 inside the leg's
-# timed steps, divided by the units (point-levels) of that launch; scaled to
-# the bench's grid by the units per launch.  Kernels that run in row chunks
-# (the learned step's networks and increments) carry bytes per unit of a
-# whole step instead (PER_STEP_UNITS).  Valid while the sources that define
-# the timed kernels are the ones captured (SHA-256 over KERNEL_SOURCES).
+# DRAM traffic per unit of every kernel, from ncu captures of the leg's timed step
+# at R2B5 L90 (dram__bytes_read.sum + dram__bytes_write.sum, one pass, every
+# launch of the step), divided by the units (point-levels) of its launches, the
+# mean over them; scaled to the bench's grid by the units per launch.  Kernels
+# that run in row chunks (the learned step's networks and increments) carry
+# bytes per unit of a whole step instead (per_step_units).  Valid while the
+# sources that define the timed kernels are the ones captured (SHA-256 over
+# KERNEL_SOURCES).
 DRAM_PER_UNIT = {
-    "sources_sha256": "1c755f8073d4233f8d10e6c746013f70051ad72effbae2380259e228a05b1090",
+    "sources_sha256": "8a020b89bb7c8015c09950cab0b5d676011c0f153a5256088b9c9cd689f71194",
     "bisections": 5, "nlev": 90,
     "legs": {
         "fp64": {
-            "diff_cell_update": 57.627, "diff_div_curl_uv": 29.152, "diff_edge_smag": 30.742,
-            "diff_edge_update": 38.763, "diff_second": 52.87, "sn_cell_div": 31.13, "sn_cell_fluxsum": 36.227,
-            "sn_cell_grad": 66.955, "sn_column_corr": 274.264, "sn_column_pred": 208.707, "sn_edge_corr": 44.137,
-            "sn_edge_flux": 42.929, "sn_edge_pred": 92.494, "va_cell_vert": 41.95, "va_cell_w": 25.65,
-            "va_edge_pre": 27.746, "va_edge_tend": 51.936},
+            "diff_cell_update": 57.136, "diff_div_curl_uv": 28.943, "diff_edge_smag": 30.935,
+            "diff_edge_update": 38.597, "diff_second": 52.546, "sn_cell_div": 23.279, "sn_cell_fluxsum": 35.805,
+            "sn_cell_grad": 66.134, "sn_column_corr": 227.942, "sn_column_pred": 192.266,
+            "sn_edge_corr": 43.869, "sn_edge_flux": 42.615, "sn_edge_pred": 92.106, "va_cell_vert": 47.147,
+            "va_cell_w": 25.233, "va_edge_pre": 27.393, "va_edge_tend": 51.744},
         "mixed": {
-            "diff_cell_update": 56.156, "diff_div_curl_uv": 10.468, "diff_edge_smag": 13.727,
-            "diff_edge_update": 28.821, "diff_second": 24.801, "mx_refresh": 20.004, "sn_cell_div": 20.767,
-            "sn_cell_fluxdiv": 34.433, "sn_cell_grad": 42.77, "sn_column_corr": 304.048, "sn_column_pred": 201.923,
-            "sn_edge_corr": 31.213, "sn_edge_pred": 47.884, "va_cell_vert": 20.033, "va_cell_w": 11.302,
-            "va_edge_pre": 11.198, "va_edge_tend": 24.854, "va_fused": 44.53},
-        # the learned step: the mixed kernels (their R2B5 figures) and its own
+            "diff_cell_update": 60.033, "diff_div_curl_uv": 10.114, "diff_edge_smag": 13.659,
+            "diff_edge_update": 28.448, "diff_second": 25.107, "mx_refresh": 19.644, "sn_cell_div": 13.166,
+            "sn_cell_fluxdiv": 33.938, "sn_cell_grad": 42.321, "sn_column_corr": 236.919,
+            "sn_column_pred": 183.447, "sn_edge_corr": 31.603, "sn_edge_pred": 48.542, "va_cell_vert": 22.825,
+            "va_cell_w": 11.033, "va_edge_pre": 11.101, "va_edge_tend": 25.051, "va_fused": 38.417},
+        # the reduced step's mixed kernels and the learned step's own
         "learned": {
-            "diff_cell_update": 56.156, "diff_div_curl_uv": 10.468, "diff_edge_smag": 13.727,
-            "diff_edge_update": 28.821, "diff_second": 24.801, "lc_apply_col": 20.923, "lc_apply_edge": 15.437,
-            "lc_col_inputs": 61.505, "lc_edge_inputs": 39.974, "lc_reduce_status": 527360.0,
-            "lc_reduce_status2": 9728.0, "mlp_gemm_tc": 12979.303, "mx_refresh": 20.004, "sn_cell_div": 20.767,
-            "sn_cell_fluxdiv": 34.433, "sn_cell_grad": 42.77, "sn_column_corr": 304.048, "sn_column_pred": 201.923,
-            "sn_edge_corr": 31.213, "sn_edge_pred": 47.884, "va_cell_vert": 20.033, "va_cell_w": 11.302,
-            "va_edge_pre": 11.198, "va_edge_tend": 24.854},
+            "diff_cell_update": 60.05, "diff_div_curl_uv": 10.153, "diff_edge_smag": 13.663,
+            "diff_edge_update": 28.502, "diff_second": 25.129, "lc_apply_col": 20.768, "lc_apply_edge": 15.192,
+            "lc_col_inputs": 61.265, "lc_edge_inputs": 39.664, "lc_reduce_status": 529152.0,
+            "lc_reduce_status2": 10752.0, "mlp_gemm_tc": 12876.15, "mx_refresh": 19.672, "sn_cell_div": 13.244,
+            "sn_cell_fluxdiv": 33.93, "sn_cell_grad": 42.394, "sn_column_corr": 237.118,
+            "sn_column_pred": 183.441, "sn_edge_corr": 31.53, "sn_edge_pred": 48.524, "va_cell_vert": 22.822,
+            "va_cell_w": 11.024, "va_edge_pre": 11.113, "va_edge_tend": 25.047}
     }}
 
 # The files whose code runs on the device in the timed steps.
@@ -400,27 +400,37 @@ def dram_measured(leg, prof, nsteps, ms_per_step, sizes, nlev, ndyn):
     stage = stage_bytes_per_step(leg, nc, ne, nv, nlev, ndyn)
     return {"bytes_per_step": b, "achieved_gbs": gbs, "peak_gbs": peak, "peak_source": src, "frac": gbs / peak,
             "stage_bytes_per_step": stage, "amplification": b / stage if stage else None,
-            "note": "per-kernel DRAM bytes per unit from one-launch ncu captures at R2B%d L%d, times the units "
+            "note": "per-kernel DRAM bytes per unit from ncu captures of a step at R2B%d L%d, times the units "
                     "and launches of this step, over the event-timed step; of %s peak"
                     % (DRAM_PER_UNIT["bisections"], DRAM_PER_UNIT["nlev"], src)}
 
 
 # FP64 instructions per unit (DADD + DMUL + DFMA) where ncu counted them
-# (`smsp__sass_thread_inst_executed_op_{dadd,dmul,dfma}_pred_on`, R2B5 L90, the
-# predictor in 8-level and the corrector in 4-level chunks): the FP64 pipe
-# issues one of any kind per slot, so the instruction rate against the pipe's
-# (half the FMA flop rate) is how busy the pipe is, whatever the mix of adds
-# and FMAs.
-FP64_INSTR_PER_UNIT = {"sn_column_pred": 56.9, "sn_column_corr": 63.5}
+# (`smsp__sass_thread_inst_executed_op_{dadd,dmul,dfma}_pred_on`, R2B5 L90), by
+# the levels per chunk that the autotuner chose: the FP64 pipe issues one of any
+# kind per slot, so the instruction rate against the pipe's (half the FMA flop
+# rate) is how busy the pipe is, whatever the mix of adds and FMAs.
+FP64_INSTR_PER_UNIT = {"sn_column_pred": {4: 58.4, 6: 56.8, 8: 56.9}, "sn_column_corr": {4: 63.5, 6: 59.3, 8: 59.0}}
+
+
+def column_chunks(launch_config):
+    """Levels per chunk of the column solve's two forms, from the library's text
+    of its launch shapes; {} in the form for small grids, which was not counted."""
+    d = dict(x.split("=") for x in launch_config.split(";")[1:])
+    if d["column_columns"] != "32":
+        return {}
+    return {"sn_column_pred": int(d["column_chunk"]), "sn_column_corr": int(d["column_corrector_chunk"])}
+
 
 # The column solve's predictor and corrector launches are one kernel (one
 # function, two forms); the roofline treats them together.
 FAMILY = {"sn_column_pred": "sn_column", "sn_column_corr": "sn_column"}
 
 
-def roofline(prof, nc, ne, nv, nlev, leg="fp64"):
+def roofline(prof, nc, ne, nv, nlev, leg="fp64", chunks=None):
     """FP64-ALU roofline of the kernel family with the largest share of the
-    step, with its HBM fraction from the captured bytes per unit."""
+    step, with its HBM fraction from the captured bytes per unit and, with the
+    column solve's chunks, its share of the FP64 pipe's instruction rate."""
     fam = {}
     for k, (n, ms) in prof.items():
         b = base_name(k)
@@ -435,8 +445,9 @@ def roofline(prof, nc, ne, nv, nlev, leg="fp64"):
     name, (n, ms, flops, units, members) = max(fam.items(), key=lambda kv: kv[1][1])
     achieved = flops / (ms / 1000.0) / 1e12
     issue = None
-    if all(m in FP64_INSTR_PER_UNIT for m in members):
-        instr = sum(FP64_INSTR_PER_UNIT[base_name(k)] * units_per_launch(k, nc, ne, nv, nlev) * prof[k][0]
+    if chunks and all(m in FP64_INSTR_PER_UNIT for m in members):
+        instr = sum(FP64_INSTR_PER_UNIT[base_name(k)][chunks[base_name(k)]]
+                    * units_per_launch(k, nc, ne, nv, nlev) * prof[k][0]
                     for k in prof if FAMILY.get(base_name(k), base_name(k)) == name)
         rate = instr / (ms / 1000.0) / 1e12
         issue = {"achieved": rate, "peak": FP64_PEAK_TFLOPS / 2, "unit": "T FP64 instructions/s",
@@ -456,7 +467,7 @@ def roofline(prof, nc, ne, nv, nlev, leg="fp64"):
             "frac": achieved / FP64_PEAK_TFLOPS, "traffic": traffic, "hbm": hbm, "fp64_issue": issue,
             "note": "FP64 algorithmic flops per launch / event-timed launch duration (CUDA events around every "
                     "launch on the library's stream); peak = nominal FP64 rate from unit counts and clock "
-                    "(1.2 TFLOP/s measured by a DFMA probe); traffic = DRAM bytes per launch from the one-kernel "
+                    "(1.2 TFLOP/s measured by a DFMA probe); traffic = DRAM bytes per launch from the "
                     "ncu captures, scaled by units; hbm = that traffic over the event time"}
 
 
@@ -811,7 +822,7 @@ def run_ours(args):
         prof, nsp = f64["prof"], f64["nsteps_prof"]
         launches_per_step = sum(n for n, _ in prof.values()) // nsp
         kernels = kernel_table(prof, nsp)
-        roof = roofline(prof, nc, ne, nv, nlev)
+        roof = roofline(prof, nc, ne, nv, nlev, chunks=column_chunks(f64["launch_config"]))
 
     mixed = {}
     for leg in ("mixed", "mixed_f64col"):

@@ -9,6 +9,10 @@ import sys
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
+CONFIG = ("va_edge_pre=128t,va_cell_vert=512,column_threads=160;column_columns=32;column_corrector_threads=160;"
+          "column_corrector_chunk=4;column_chunk=8")
+
+
 def _full(B):
     """A record of a default run: kernel tables of the real kernels, long numbers, notes."""
     x = 1234.567890123456789
@@ -25,7 +29,7 @@ def _full(B):
         "metric": B.METRIC, "value": x / 100, "unit": "steps/s", "n_gpus": 8, "steps": 100, "warmup": 100,
         "ms_per_step": x, "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64",
         "data": "synthetic", "config": B.config_dict("fp64"), "sdpd": x, "hbm": dict(hbm, stage_frac=x),
-        "hbm_measured": hbm, "roofline": B.roofline(prof, nc, ne, nv, 90), "kernels": B.kernel_table(prof, 2),
+        "hbm_measured": hbm, "roofline": B.roofline(prof, nc, ne, nv, 90, chunks=B.column_chunks(CONFIG)), "kernels": B.kernel_table(prof, 2),
         "autotuned_launch_config": "a" * 600, "steps_compared": 240, "mixed": leg, "mixed_f64col": leg,
         "mixed_learned": learned, "mountain_r2b7": {"config": {}, "fp64": leg, "mixed": leg, "mixed_learned": learned},
         "e2e": B.end_to_end([x / 1000] * 9 + [x / 500], 1536163840),
@@ -74,3 +78,19 @@ def test_the_end_to_end_rate_counts_every_step():
     assert abs(e["value"] - 10 / (0.8 + 0.165 + 0.164)) < 1e-12
     assert abs(e["median_value"] - 10.0) < 1e-12
     assert e["h2d_bytes_per_step"] == e["d2h_bytes_per_step"] == 7 and e["step_ms"][-2:] == [165.0, 164.0]
+
+
+def test_fp64_instructions_are_those_of_the_chunks_that_ran():
+    if ROOT not in sys.path:
+        sys.path.insert(0, ROOT)
+    B = importlib.import_module("bench")
+    nc, ne, nv = 327680, 491520, 163842
+    prof = {"sn_column_pred": (5, 10.0), "sn_column_corr": (5, 12.0)}
+    t = B.FP64_INSTR_PER_UNIT
+    for corr in (4, 6, 8):
+        text = CONFIG.replace("corrector_chunk=4", "corrector_chunk=%d" % corr)
+        r = B.roofline(prof, nc, ne, nv, 90, chunks=B.column_chunks(text))
+        want = (t["sn_column_pred"][8] + t["sn_column_corr"][corr]) * nc * 90 * 5 / 0.022 / 1e12
+        assert abs(r["fp64_issue"]["achieved"] - want) < 1e-12 * want
+    assert B.column_chunks(CONFIG.replace("columns=32", "columns=16")) == {}
+    assert B.roofline(prof, nc, ne, nv, 90, chunks={})["fp64_issue"] is None
